@@ -31,7 +31,9 @@ struct scw_fno_s {
   int step = 0;
   float q_cal = 0.f;
 
-  void* D = nullptr;        // [Kc][P]
+  void* D = nullptr;        // [2 n_ind][P]
+  int2* modes = nullptr;    // [n_ind] independent modes of a real input's DFT (dft_independent_modes)
+  int n_ind = 0;
   void* E = nullptr;        // [P][Kp]
   void* Vcf[9] = {};        // [Bmax][C][P]
   void* Vcl[9] = {};        // [Bmax][P][C]
@@ -55,7 +57,7 @@ struct scw_fno_s {
   int* d_err = nullptr;
   uint64_t timeout_ns = 2000000000ull;
 
-  CUtensorMap map_Vcf[9], map_dZcf[2], map_D, map_E, map_Wh, map_GVh;
+  CUtensorMap map_Vcf[9], map_dZcf[2], map_D[kDftTileCount], map_E, map_Wh, map_GVh;
   // 1x1-convolution operands: channel-first activations read MN-major (3D maps), W and W^T
   CUtensorMap map_Vx[8], map_dZx[2], map_W[8], map_WT[8];
 
@@ -108,9 +110,10 @@ static double uniform_pm1(unsigned long long seed, unsigned long long i) {
   return 2.0 * ((double)(z >> 11) * (1.0 / 9007199254740992.0)) - 1.0;
 }
 
-static int dft_splits(const scw_fno_s* f, int B, int BN) {
-  if (f->bf16 && BN == 256) return 1;  // the persistent GEMM form: deep pipeline, no K splits
-  const int tiles = ((B * C + 127) / 128) * ((f->Kc + BN - 1) / BN);
+// K splits of the FP32 (SIMT) truncated DFT; the tensor-core form never splits K
+static int dft_splits(const scw_fno_s* f, int B) {
+  if (f->bf16) return 1;
+  const int tiles = ((B * C + 127) / 128) * ((2 * f->n_ind + 31) / 32);
   int ks = std::max(1, (2 * 152) / std::max(1, tiles));
   ks = std::min(ks, kMaxSplit);
   ks = std::min(ks, std::max(1, f->P / 64 / 4));  // at least 4 K blocks per split
@@ -124,8 +127,6 @@ static int dw_splits(const scw_fno_s* f, int B) {
   ks = std::min(ks, std::max(1, f->P / 64 / 4));
   return ks;
 }
-
-static int dft_bn(const scw_fno_s* f) { return f->Kc >= 256 ? 256 : (f->Kc >= 128 ? 128 : (f->Kc >= 64 ? 64 : 32)); }
 
 // record timing event i (created on first use)
 static cudaError_t mark(scw_fno_s* f, size_t i) {
@@ -210,19 +211,19 @@ static scw_status forward(scw_fno_s* f, const float2* n, int B, bool keep_z, cud
   const long long vstride = ld * (f->Kc / 2);                 // complex elements per split
   const float inv_n2 = 1.f / ((float)f->N * (float)f->N);
   for (int l = 0; l < f->L; ++l) {
-    const int bn = dft_bn(f);
-    const int ks = dft_splits(f, B, bn);
+    const int ks = dft_splits(f, B), Kd = 2 * f->n_ind;
     EpiArgs ea{};
     ea.alpha = 1.f;
     ea.rows = BC;
-    ea.cols = f->Kc;
+    ea.cols = Kd;
+    ea.modes = f->modes;
     ea.out = f->Vh[l];
     ea.ld = ld;
     ea.split_stride = vstride;
-    cudaError_t e = f->bf16 ? launch_gemm_tc(EPI_MODES, bn, f->map_Vcf[l], f->map_D, f->map_D, f->map_D, ea, BC,
-                                             f->Kc, f->P, ks, f->d_err, f->timeout_ns, st)
+    cudaError_t e = f->bf16 ? launch_dft_tc(f->map_Vcf[l], f->map_D, nullptr, ea, nullptr, BC, Kd, f->P, f->d_err,
+                                            f->timeout_ns, st)
                             : launch_gemm_simt(EPI_MODES, static_cast<const float*>(f->Vcf[l]), f->P,
-                                               static_cast<const float*>(f->D), f->P, ea, BC, f->Kc, f->P, ks, st);
+                                               static_cast<const float*>(f->D), f->P, ea, BC, Kd, f->P, ks, st);
     FNO_TRY(launch_ok(f, e, "truncated DFT", CAT_DFT, 2.0 * BC * f->Kc * f->P));
     // Wh carries the inverse transform's 1/N^2 so that the 1x1 convolution can share its accumulator
     if constexpr (std::is_same<T, __nv_bfloat16>::value)
@@ -315,12 +316,12 @@ static scw_status forward_backward(scw_fno_s* f, const float2* n, const float2* 
   const long long mix_w = (long long)f->m * f->m * C * C * 2;
   int cur = 0;
   for (int l = f->L - 1; l >= 0; --l) {
-    const int bn = dft_bn(f);
-    const int ks = dft_splits(f, B, bn);
+    const int ks = dft_splits(f, B), Kd = 2 * f->n_ind;
     EpiArgs ea{};
     ea.alpha = 1.f / ((float)f->N * (float)f->N);
     ea.rows = BC;
-    ea.cols = f->Kc;
+    ea.cols = Kd;
+    ea.modes = f->modes;
     ea.out = f->GWh;
     ea.ld = ld;
     ea.split_stride = vstride;
@@ -330,27 +331,20 @@ static scw_status forward_backward(scw_fno_s* f, const float2* n, const float2* 
     ew.rows = BC;
     ew.B = B;
     ew.out = f->part_dw[l];
-    // at 2 m^2 = 512 kept-mode columns both products run in one kernel that reads dZ once (the two
-    // column tiles of the DFT each take one half of the pixels of dW: two partials)
-    const bool fused = f->bf16 && bn == 256 && ks == 1 && f->Kc == 512 && P % 128 == 0;
-    const int kw = fused ? 2 : dw_splits(f, B);
+    // BF16: both products run in one kernel that reads dZ once (two column tiles of the DFT each take one
+    // half of the pixels of dW: two partials)
+    const int kw = f->bf16 ? 2 : dw_splits(f, B);
     ew.splits = kw;
-    if (fused) {
-      e = launch_gemm_dft_dw(f->map_dZcf[cur], f->map_D, f->map_Vcf[l], ea, ew, BC, f->Kc, P, f->d_err,
-                             f->timeout_ns, st);
+    if (f->bf16) {
+      e = launch_dft_tc(f->map_dZcf[cur], f->map_D, &f->map_Vcf[l], ea, &ew, BC, Kd, P, f->d_err, f->timeout_ns, st);
       FNO_TRY(launch_ok(f, e, "truncated DFT of dZ and weight gradient", CAT_DFT,
                         2.0 * BC * f->Kc * P + 2.0 * BC * C * P));
     } else {
-      e = f->bf16 ? launch_gemm_tc(EPI_MODES, bn, f->map_dZcf[cur], f->map_D, f->map_D, f->map_D, ea, BC, f->Kc, P,
-                                   ks, f->d_err, f->timeout_ns, st)
-                  : launch_gemm_simt(EPI_MODES, static_cast<const float*>(f->dZcf[cur]), P,
-                                     static_cast<const float*>(f->D), P, ea, BC, f->Kc, P, ks, st);
+      e = launch_gemm_simt(EPI_MODES, static_cast<const float*>(f->dZcf[cur]), P, static_cast<const float*>(f->D), P,
+                           ea, BC, Kd, P, ks, st);
       FNO_TRY(launch_ok(f, e, "truncated DFT of dZ", CAT_DFT, 2.0 * BC * f->Kc * P));
-      e = f->bf16 ? launch_gemm_tc(EPI_DW, 128, f->map_dZcf[cur], f->map_Vcf[l], f->map_D, f->map_D, ew, groups * 128,
-                                   groups * 128, P, kw, f->d_err, f->timeout_ns, st)
-                  : launch_gemm_simt(EPI_DW, static_cast<const float*>(f->dZcf[cur]), P,
-                                     static_cast<const float*>(f->Vcf[l]), P, ew, groups * 128, groups * 128, P, kw,
-                                     st);
+      e = launch_gemm_simt(EPI_DW, static_cast<const float*>(f->dZcf[cur]), P, static_cast<const float*>(f->Vcf[l]), P,
+                           ew, groups * 128, groups * 128, P, kw, st);
       FNO_TRY(launch_ok(f, e, "weight gradient", CAT_DW, 2.0 * BC * C * P));
     }
     reduce_into(segs, f->part_dw[l], groups * kw * 4, C * C, C * C, f->grad + f->off_W[l]);
@@ -500,7 +494,10 @@ scw_status scw_surrogate_create(const scw_fno_desc* d, scw_fno_t* out) {
   A((void**)&f->adam_m, f->n_params * 4);
   A((void**)&f->adam_v, f->n_params * 4);
   A(&f->wcopy, f->n_params * esz);
-  A(&f->D, (size_t)f->Kc * P * esz);
+  std::vector<int2> modes;
+  f->n_ind = dft_independent_modes(f->m, modes);
+  A(&f->D, (size_t)2 * f->n_ind * P * esz);
+  A((void**)&f->modes, (size_t)f->n_ind * sizeof(int2));
   A(&f->E, P * f->Kp * esz);
   for (int l = 0; l <= f->L; ++l) {
     A(&f->Vcf[l], act);
@@ -544,10 +541,12 @@ scw_status scw_surrogate_create(const scw_fno_desc* d, scw_fno_t* out) {
   if (e == cudaSuccess) e = cudaMemsetAsync(f->Wh, 0, Bm * C * f->Kp * esz, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(f->GVh, 0, Bm * C * f->Kp * esz, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(f->d_err, 0, 4, st);
+  if (e == cudaSuccess) e = cudaMemcpy(f->modes, modes.data(), modes.size() * sizeof(int2), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
     e = f->bf16 ? launch_tables<__nv_bfloat16>(static_cast<__nv_bfloat16*>(f->D), static_cast<__nv_bfloat16*>(f->E),
-                                               f->N, f->m, f->Kp, st)
-                : launch_tables<float>(static_cast<float*>(f->D), static_cast<float*>(f->E), f->N, f->m, f->Kp, st);
+                                               f->modes, f->n_ind, f->N, f->m, f->Kp, st)
+                : launch_tables<float>(static_cast<float*>(f->D), static_cast<float*>(f->E), f->modes, f->n_ind, f->N,
+                                       f->m, f->Kp, st);
   std::vector<float> init((size_t)f->n_params, 0.f);
   {
     auto fill = [&](long long off, long long count, double scale) {
@@ -576,7 +575,8 @@ scw_status scw_surrogate_create(const scw_fno_desc* d, scw_fno_t* out) {
   }
   if (f->bf16) {
     const long long BCm = (long long)f->Bmax * C;
-    s = make_map_bf16(&f->map_D, f->D, f->P, f->Kc, f->P, dft_bn(f));
+    for (int i = 0; i < kDftTileCount && s == SCW_OK; ++i)
+      s = make_map_bf16(&f->map_D[i], f->D, f->P, 2 * f->n_ind, f->P, kDftTiles[i]);
     if (s == SCW_OK) s = make_map_bf16(&f->map_E, f->E, f->Kp, f->P, f->Kp, 128);
     if (s == SCW_OK) s = make_map_bf16(&f->map_Wh, f->Wh, f->Kp, BCm, f->Kp, 256);
     if (s == SCW_OK) s = make_map_bf16(&f->map_GVh, f->GVh, f->Kp, BCm, f->Kp, 256);

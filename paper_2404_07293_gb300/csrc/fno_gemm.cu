@@ -23,12 +23,12 @@
 // error word, lets issued copies and MMAs land, frees its tensor memory and exits.
 //
 // The products (N = pixels per sample, m = kept modes per axis, C = 32 channels):
-//   truncated DFT        Vh [B C][2 m^2]  = V_cf [B C][N^2] . D [2 m^2][N^2]^T, stored
-//                        mode-major as complex Vh[mode][B C]                     (EPI_MODES)
+//   truncated DFT        Vh [B C][modes]  = V_cf [B C][N^2] . D [2 x independent modes][N^2]^T, stored
+//                        mode-major as complex Vh[mode][B C]       (EPI_MODES; tensor cores: fno_dft.cu)
 //   inverse + 1x1 conv   Z^T [N^2][B C]   = E [N^2][Kp] . Wh [B C][Kp]^T + V_cl W^T,
 //                        then + c and GELU in the epilogue                       (EPI_LAYER_FWD)
 //   backward of both     dV^T [N^2][B C]  = E . GVh^T + dZ_cl W, * GELU'(Z)      (EPI_LAYER_BWD)
-//   weight gradient      dW = sum_b dZ_b V_b^T over pixels, 4 samples per tile  (EPI_DW)
+//   weight gradient      dW = sum_b dZ_b V_b^T over pixels, 4 samples per tile  (EPI_DW; tensor cores: fno_dft.cu)
 // The field synthesis at arbitrary lateral points uses the same engine for its
 // product over the orders, E[point][(plane, component)] (EPI_FIELD, split-BF16
 // operands along a tripled K; see scw_points.cu).
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_tc_kernel(const __grid_c
                                                                   int* err, uint64_t timeout_ns) {
   using Cfg = GemmCfg<BN>;
   constexpr int STAGES = Cfg::STAGES;
-  static_assert(EPI == EPI_MODES || EPI == EPI_DW || EPI == EPI_FIELD, "layer products run persistent");
+  static_assert(EPI == EPI_FIELD, "the DFTs have their own kernel, the layer products run persistent");
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[STAGES];
   __shared__ __align__(8) uint64_t empty_bar[STAGES];
@@ -83,10 +83,8 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_tc_kernel(const __grid_c
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // EPI_FIELD walks the column tiles fastest, so the CTAs that share a row tile of A run together
-  constexpr bool NFAST = (EPI == EPI_FIELD);
-  const int m0 = (NFAST ? blockIdx.y : blockIdx.x) * 128;
-  const int n0 = (EPI == EPI_DW) ? m0 : (NFAST ? blockIdx.x : blockIdx.y) * BN;
+  // the column tiles run fastest, so the CTAs that share a row tile of A run together
+  const int m0 = blockIdx.y * 128, n0 = blockIdx.x * BN;
   const int kb0 = blockIdx.z * kper;
   const int nkb = max(0, min(K / 64 - kb0, kper));
   const int total = nkb;
@@ -113,46 +111,48 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_tc_kernel(const __grid_c
   ptx::tc_fence_after();
   const uint32_t tmem = tmem_base_s;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ---------------- TMA producer ----------------
+    const uint32_t leader = ptx::elect_one();
     int st = 0, issued = 0;
     uint32_t ph = 0;
-    for (int i = 0; i < total && !abort_s; ++i) {
-      if (!ptx::mbar_wait(ptx::smem_u32(&empty_bar[st]), ph ^ 1u, deadline)) {
-        atomicOr(err, DEV_ERR_TIMEOUT_EMPTY);
+    for (int i = 0; i < total && !ptx::warp_any(abort_s); ++i) {
+      if (!ptx::mbar_wait_warp(ptx::smem_u32(&empty_bar[st]), ph ^ 1u, deadline)) {
+        if (leader) atomicOr(err, DEV_ERR_TIMEOUT_EMPTY);
         abort_s = 1;
         break;
       }
       const uint32_t fb = ptx::smem_u32(&full_bar[st]);
       const uint32_t sa = ptx::smem_u32(smem + (size_t)st * Cfg::STAGE);
-      ptx::mbar_arrive_expect_tx(fb, Cfg::STAGE);
+      ptx::mbar_arrive_expect_tx(fb, Cfg::STAGE, leader);
       const int kc = (kb0 + i) * 64;
-      ptx::tma_load_2d(sa, &mA, kc, m0, fb);
-      ptx::tma_load_2d(sa + Cfg::A_BYTES, &mB, kc, n0, fb);
+      ptx::tma_load_2d(sa, &mA, kc, m0, fb, leader);
+      ptx::tma_load_2d(sa + Cfg::A_BYTES, &mB, kc, n0, fb, leader);
       ++issued;
       if (++st == STAGES) {
         st = 0;
         ph ^= 1u;
       }
     }
-    if (abort_s) {
+    if (ptx::warp_any(abort_s)) {
       const uint64_t d2 = ptx::drain_deadline(timeout_ns);
       for (int back = 1; back <= STAGES && back <= issued; ++back) {
         const int i = issued - back;
-        if (!ptx::mbar_wait(ptx::smem_u32(&full_bar[i % STAGES]), (uint32_t)(i / STAGES) & 1u, d2)) {
-          atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
+        if (!ptx::mbar_wait_warp(ptx::smem_u32(&full_bar[i % STAGES]), (uint32_t)(i / STAGES) & 1u, d2)) {
+          if (leader) atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
           break;
         }
       }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------- tcgen05.mma issuer ----------------
+    const uint32_t leader = ptx::elect_one();
     constexpr uint32_t idesc = ptx::idesc_f16(true, 128, BN);
     int st = 0;
     uint32_t ph = 0;
-    for (int i = 0; i < total && !abort_s; ++i) {
-      if (!ptx::mbar_wait(ptx::smem_u32(&full_bar[st]), ph, deadline)) {
-        atomicOr(err, DEV_ERR_TIMEOUT_FULL);
+    for (int i = 0; i < total && !ptx::warp_any(abort_s); ++i) {
+      if (!ptx::mbar_wait_warp(ptx::smem_u32(&full_bar[st]), ph, deadline)) {
+        if (leader) atomicOr(err, DEV_ERR_TIMEOUT_FULL);
         abort_s = 1;
         break;
       }
@@ -162,20 +162,20 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_tc_kernel(const __grid_c
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
         const uint64_t o = (uint64_t)(2 * kk);  // 16 elements = 32 bytes, in 16-byte units
-        ptx::mma_f16(tmem, da + o, db + o, idesc, (i > 0 || kk > 0) ? 1u : 0u);
+        ptx::mma_f16(tmem, da + o, db + o, idesc, (i > 0 || kk > 0) ? 1u : 0u, leader);
       }
-      ptx::mma_commit(ptx::smem_u32(&empty_bar[st]));
+      ptx::mma_commit(ptx::smem_u32(&empty_bar[st]), leader);
       if (++st == STAGES) {
         st = 0;
         ph ^= 1u;
       }
     }
-    if (!abort_s) {
-      ptx::mma_commit(ptx::smem_u32(&acc_bar));
+    if (!ptx::warp_any(abort_s)) {
+      ptx::mma_commit(ptx::smem_u32(&acc_bar), leader);
     } else {
-      ptx::mma_commit(ptx::smem_u32(&drain_bar));
-      if (!ptx::mbar_wait(ptx::smem_u32(&drain_bar), 0u, ptx::drain_deadline(timeout_ns)))
-        atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
+      ptx::mma_commit(ptx::smem_u32(&drain_bar), leader);
+      if (!ptx::mbar_wait_warp(ptx::smem_u32(&drain_bar), 0u, ptx::drain_deadline(timeout_ns)))
+        if (leader) atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
     }
   } else if (warp >= 2) {
     // ---------------- epilogue ----------------
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_tc_kernel(const __grid_c
       ptx::tc_fence_after();
       const int row = m0 + grp * 32 + lane;
       const uint32_t lane_addr = tmem + ((uint32_t)(grp * 32) << 16);
-      const int col_end = (EPI == EPI_DW) ? n0 + 128 : ea.cols;
+      const int col_end = ea.cols;
 #pragma unroll 1
       for (int c = half; c < BN / 32; c += 2) {
         if (n0 + 32 * c >= col_end) break;  // warp-uniform
@@ -315,9 +315,8 @@ __global__ void __launch_bounds__(kLayerThreads, 1) gemm_layer_persistent(const 
   constexpr bool SEG2 = (EPI == EPI_LAYER_FWD || EPI == EPI_LAYER_BWD);
   const int n_tasks = m_tiles * n_tiles;
   // the layer products walk the row tiles fastest (CTAs in flight share a Wh / GVh tile); the
-  // field product and the truncated DFT walk the column tiles fastest (they share a row tile of
-  // the points table / the activations)
-  constexpr bool NFAST = (EPI == EPI_FIELD || EPI == EPI_MODES);
+  // field product walks the column tiles fastest (they share a row tile of the points table)
+  constexpr bool NFAST = (EPI == EPI_FIELD);
   auto tile_m0 = [&](int t) { return (NFAST ? t / n_tiles : t % m_tiles) * 128; };
   auto tile_n0 = [&](int t) { return (NFAST ? t % n_tiles : t / m_tiles) * BN; };
   // samples of a tile whose 1x1 convolution runs as an extra K segment, and the operand stages
@@ -356,33 +355,34 @@ __global__ void __launch_bounds__(kLayerThreads, 1) gemm_layer_persistent(const 
   ptx::tc_fence_after();
   const uint32_t tmem = tmem_base_s;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ---------------- TMA producer ----------------
+    const uint32_t leader = ptx::elect_one();
     int st = 0, issued = 0;
     uint32_t ph = 0;
-    for (int t = blockIdx.x; t < n_tasks && !abort_s; t += gridDim.x) {
+    for (int t = blockIdx.x; t < n_tasks && !ptx::warp_any(abort_s); t += gridDim.x) {
       const int m0 = tile_m0(t), n0 = tile_n0(t);
       const int total = nkb + tile_ngrp(n0);
-      for (int i = 0; i < total && !abort_s; ++i) {
-        if (!ptx::mbar_wait(ptx::smem_u32(&empty_bar[st]), ph ^ 1u, deadline)) {
-          atomicOr(err, DEV_ERR_TIMEOUT_EMPTY);
+      for (int i = 0; i < total && !ptx::warp_any(abort_s); ++i) {
+        if (!ptx::mbar_wait_warp(ptx::smem_u32(&empty_bar[st]), ph ^ 1u, deadline)) {
+          if (leader) atomicOr(err, DEV_ERR_TIMEOUT_EMPTY);
           abort_s = 1;
           break;
         }
         const uint32_t fb = ptx::smem_u32(&full_bar[st]);
         const uint32_t sa = ptx::smem_u32(smem + (size_t)st * kLayerStage);
         if (i < nkb) {
-          ptx::mbar_arrive_expect_tx(fb, kLayerStage);
-          ptx::tma_load_2d(sa, &mA, i * 64, m0, fb);
-          ptx::tma_load_2d(sa + A_BYTES, &mB, i * 64, n0, fb);
+          ptx::mbar_arrive_expect_tx(fb, kLayerStage, leader);
+          ptx::tma_load_2d(sa, &mA, i * 64, m0, fb, leader);
+          ptx::tma_load_2d(sa + A_BYTES, &mB, i * 64, n0, fb, leader);
         } else {
           // X_s for samples smp0 .. smp0 + kSeg2Samples - 1 (pixels m0 .. m0 + 63, then
           // m0 + 64 .. m0 + 127; the pixel count is a multiple of 128), then W
           const int smp0 = n0 / C + kSeg2Samples * (i - nkb);
-          ptx::mbar_arrive_expect_tx(fb, kSeg2Bytes);
-          ptx::tma_load_3d(sa, &mA2, m0, 0, smp0, fb);
-          ptx::tma_load_3d(sa + kSeg2HalfBytes, &mA2, m0 + 64, 0, smp0, fb);
-          ptx::tma_load_2d(sa + 2u * kSeg2HalfBytes, &mW, 0, 0, fb);
+          ptx::mbar_arrive_expect_tx(fb, kSeg2Bytes, leader);
+          ptx::tma_load_3d(sa, &mA2, m0, 0, smp0, fb, leader);
+          ptx::tma_load_3d(sa + kSeg2HalfBytes, &mA2, m0 + 64, 0, smp0, fb, leader);
+          ptx::tma_load_2d(sa + 2u * kSeg2HalfBytes, &mW, 0, 0, fb, leader);
         }
         ++issued;
         if (++st == STAGES) {
@@ -391,37 +391,38 @@ __global__ void __launch_bounds__(kLayerThreads, 1) gemm_layer_persistent(const 
         }
       }
     }
-    if (abort_s) {
+    if (ptx::warp_any(abort_s)) {
       const uint64_t d2 = ptx::drain_deadline(timeout_ns);
       for (int back = 1; back <= STAGES && back <= issued; ++back) {
         const int i = issued - back;
-        if (!ptx::mbar_wait(ptx::smem_u32(&full_bar[i % STAGES]), (uint32_t)(i / STAGES) & 1u, d2)) {
-          atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
+        if (!ptx::mbar_wait_warp(ptx::smem_u32(&full_bar[i % STAGES]), (uint32_t)(i / STAGES) & 1u, d2)) {
+          if (leader) atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
           break;
         }
       }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------- tcgen05.mma issuer ----------------
+    const uint32_t leader = ptx::elect_one();
     constexpr uint32_t idesc = ptx::idesc_f16(true, 128, BN);
     constexpr uint32_t idesc32 = ptx::idesc_f16(true, 128, 32, true);  // A (activations) MN-major
     int st = 0, lt = 0;
     uint32_t ph = 0;
-    for (int t = blockIdx.x; t < n_tasks && !abort_s; t += gridDim.x, ++lt) {
+    for (int t = blockIdx.x; t < n_tasks && !ptx::warp_any(abort_s); t += gridDim.x, ++lt) {
       const int n0 = tile_n0(t);
       const int nseg = tile_nseg(n0);
       const int total = nkb + tile_ngrp(n0);
       const int acc = lt & 1;
-      if (!ptx::mbar_wait(ptx::smem_u32(&acce_bar[acc]), ((uint32_t)(lt >> 1) & 1u) ^ 1u, deadline)) {
-        atomicOr(err, DEV_ERR_TIMEOUT_ACCUM);
+      if (!ptx::mbar_wait_warp(ptx::smem_u32(&acce_bar[acc]), ((uint32_t)(lt >> 1) & 1u) ^ 1u, deadline)) {
+        if (leader) atomicOr(err, DEV_ERR_TIMEOUT_ACCUM);
         abort_s = 1;
         break;
       }
       ptx::tc_fence_after();
       const uint32_t d_tmem = tmem + (uint32_t)(acc * BN);
       for (int i = 0; i < total; ++i) {
-        if (!ptx::mbar_wait(ptx::smem_u32(&full_bar[st]), ph, deadline)) {
-          atomicOr(err, DEV_ERR_TIMEOUT_FULL);
+        if (!ptx::mbar_wait_warp(ptx::smem_u32(&full_bar[st]), ph, deadline)) {
+          if (leader) atomicOr(err, DEV_ERR_TIMEOUT_FULL);
           abort_s = 1;
           break;
         }
@@ -432,7 +433,7 @@ __global__ void __launch_bounds__(kLayerThreads, 1) gemm_layer_persistent(const 
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) {
             const uint64_t o = (uint64_t)(2 * kk);
-            ptx::mma_f16(d_tmem, da + o, db + o, idesc, (i > 0 || kk > 0) ? 1u : 0u);
+            ptx::mma_f16(d_tmem, da + o, db + o, idesc, (i > 0 || kk > 0) ? 1u : 0u, leader);
           }
         } else {
           const int s0 = kSeg2Samples * (i - nkb);
@@ -443,22 +444,22 @@ __global__ void __launch_bounds__(kLayerThreads, 1) gemm_layer_persistent(const 
             const uint32_t d = d_tmem + (uint32_t)(C * (s0 + j));
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk)
-              ptx::mma_f16(d, da + (uint64_t)(kk * (2048 >> 4)), db + (uint64_t)(2 * kk), idesc32, 1u);
+              ptx::mma_f16(d, da + (uint64_t)(kk * (2048 >> 4)), db + (uint64_t)(2 * kk), idesc32, 1u, leader);
           }
         }
-        ptx::mma_commit(ptx::smem_u32(&empty_bar[st]));
+        ptx::mma_commit(ptx::smem_u32(&empty_bar[st]), leader);
         if (++st == STAGES) {
           st = 0;
           ph ^= 1u;
         }
       }
-      if (abort_s) break;
-      ptx::mma_commit(ptx::smem_u32(&accf_bar[acc]));
+      if (ptx::warp_any(abort_s)) break;
+      ptx::mma_commit(ptx::smem_u32(&accf_bar[acc]), leader);
     }
-    if (abort_s) {
-      ptx::mma_commit(ptx::smem_u32(&drain_bar));
-      if (!ptx::mbar_wait(ptx::smem_u32(&drain_bar), 0u, ptx::drain_deadline(timeout_ns)))
-        atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
+    if (ptx::warp_any(abort_s)) {
+      ptx::mma_commit(ptx::smem_u32(&drain_bar), leader);
+      if (!ptx::mbar_wait_warp(ptx::smem_u32(&drain_bar), 0u, ptx::drain_deadline(timeout_ns)))
+        if (leader) atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
     }
   } else if (warp >= 2) {
     // ---------------- epilogue ----------------
@@ -587,237 +588,9 @@ static cudaError_t launch_tc_t(const CUtensorMap& mA, const CUtensorMap& mB, con
   if (e != cudaSuccess) return e;
   const int nkb = K / 64;
   const int kper = (nkb + splits - 1) / splits;
-  const dim3 grid = EPI == EPI_FIELD ? dim3((N + BN - 1) / BN, (M + 127) / 128, splits)
-                                     : dim3((M + 127) / 128, EPI == EPI_DW ? 1 : (N + BN - 1) / BN, splits);
+  const dim3 grid((N + BN - 1) / BN, (M + 127) / 128, splits);
   if (grid.y > 65535u) return cudaErrorInvalidValue;
   gemm_tc_kernel<BN, EPI><<<grid, kGemmThreads, Cfg::SMEM, st>>>(mA, mB, mA2, mW, ea, K, kper, err, timeout_ns);
-  return cudaGetLastError();
-}
-
-// ---- backward truncated DFT of dZ fused with the weight gradient dW = sum_b dZ_b V_b^T ----
-// Both products read dZ (channel-first, rows (b, o), K = pixels) as A. Tile (m0, n0) of the DFT
-// (2m^2 = 512 output columns, two column tiles of 256) also multiplies, over one half of K (the
-// first half for n0 = 0, the second for n0 = 256), its 128 rows of dZ by the same 128 rows of V
-// (rows (b, i), a third operand in the stage) into a 128-column accumulator beside the DFT's; the
-// diagonal 32 x 32 blocks are the four samples' dW_b partials (K half = split 0 or 1). dZ is then
-// read once per layer instead of twice. Stages: A 16 KB + D 32 KB + V 16 KB, three in flight.
-// One accumulator pair per CTA (no double buffering: at batch <= 256 every CTA has one tile).
-constexpr int kDwStages = 3;
-constexpr uint32_t kDwStage = 128u * 128u + 256u * 128u + 128u * 128u;
-constexpr uint32_t kDwSmem = kDwStages * kDwStage + 1024u;
-
-__global__ void __launch_bounds__(kLayerThreads, 1) gemm_dft_dw_kernel(const __grid_constant__ CUtensorMap mA,
-                                                                      const __grid_constant__ CUtensorMap mB,
-                                                                      const __grid_constant__ CUtensorMap mV,
-                                                                      const __grid_constant__ EpiArgs ea,
-                                                                      const __grid_constant__ EpiArgs ew, int K,
-                                                                      int m_tiles, int* err, uint64_t timeout_ns) {
-  constexpr int BN = 256, STAGES = kDwStages, n_tiles = 2;
-  constexpr uint32_t A_BYTES = 128u * 128u, B_BYTES = 256u * 128u;
-  extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full_bar[STAGES];
-  __shared__ __align__(8) uint64_t empty_bar[STAGES];
-  __shared__ __align__(8) uint64_t accf_bar;
-  __shared__ __align__(8) uint64_t acce_bar;
-  __shared__ __align__(8) uint64_t drain_bar;
-  __shared__ uint32_t tmem_base_s;
-  __shared__ volatile int abort_s;
-
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_tasks = m_tiles * n_tiles;
-  const int nkb = K / 64, half = nkb / 2;  // K blocks; the dW half of tile (m, n): [n half, (n + 1) half)
-  const uint64_t deadline = ptx::globaltimer() + timeout_ns;
-  // column tiles fastest: the two tiles of a row tile run side by side and share its dZ rows in L2
-  auto tile_m0 = [&](int t) { return (t / n_tiles) * 128; };
-  auto tile_n = [&](int t) { return t % n_tiles; };
-
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < STAGES; ++i) {
-      ptx::mbar_init(ptx::smem_u32(&full_bar[i]), 1);
-      ptx::mbar_init(ptx::smem_u32(&empty_bar[i]), 1);
-    }
-    ptx::mbar_init(ptx::smem_u32(&accf_bar), 1);
-    ptx::mbar_init(ptx::smem_u32(&acce_bar), kLayerEpiWarps);
-    ptx::mbar_init(ptx::smem_u32(&drain_bar), 1);
-    abort_s = 0;
-    ptx::fence_mbar_init();
-    ptx::prefetch_tensormap(&mA);
-    ptx::prefetch_tensormap(&mB);
-    ptx::prefetch_tensormap(&mV);
-  }
-  if (warp == 0) {
-    ptx::tmem_alloc(ptx::smem_u32(&tmem_base_s), 512);  // DFT columns [0, 256), dW columns [256, 384)
-    ptx::tmem_relinquish();
-  }
-  ptx::tc_fence_before();
-  __syncthreads();
-  ptx::tc_fence_after();
-  const uint32_t tmem = tmem_base_s;
-
-  if (warp == 0 && lane == 0) {
-    // ---------------- TMA producer ----------------
-    int st = 0, issued = 0;
-    uint32_t ph = 0;
-    for (int t = blockIdx.x; t < n_tasks && !abort_s; t += gridDim.x) {
-      const int m0 = tile_m0(t), n = tile_n(t);
-      for (int i = 0; i < nkb && !abort_s; ++i) {
-        if (!ptx::mbar_wait(ptx::smem_u32(&empty_bar[st]), ph ^ 1u, deadline)) {
-          atomicOr(err, DEV_ERR_TIMEOUT_EMPTY);
-          abort_s = 1;
-          break;
-        }
-        const bool dw = i >= n * half && i < (n + 1) * half;
-        const uint32_t fb = ptx::smem_u32(&full_bar[st]);
-        const uint32_t sa = ptx::smem_u32(smem + (size_t)st * kDwStage);
-        ptx::mbar_arrive_expect_tx(fb, A_BYTES + B_BYTES + (dw ? A_BYTES : 0u));
-        ptx::tma_load_2d(sa, &mA, i * 64, m0, fb);
-        ptx::tma_load_2d(sa + A_BYTES, &mB, i * 64, n * BN, fb);
-        if (dw) ptx::tma_load_2d(sa + A_BYTES + B_BYTES, &mV, i * 64, m0, fb);
-        ++issued;
-        if (++st == STAGES) {
-          st = 0;
-          ph ^= 1u;
-        }
-      }
-    }
-    if (abort_s) {
-      const uint64_t d2 = ptx::drain_deadline(timeout_ns);
-      for (int back = 1; back <= STAGES && back <= issued; ++back) {
-        const int i = issued - back;
-        if (!ptx::mbar_wait(ptx::smem_u32(&full_bar[i % STAGES]), (uint32_t)(i / STAGES) & 1u, d2)) {
-          atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
-          break;
-        }
-      }
-    }
-  } else if (warp == 1 && lane == 0) {
-    // ---------------- tcgen05.mma issuer ----------------
-    constexpr uint32_t idesc = ptx::idesc_f16(true, 128, BN);
-    constexpr uint32_t idesc_dw = ptx::idesc_f16(true, 128, 128);
-    int st = 0, lt = 0;
-    uint32_t ph = 0;
-    for (int t = blockIdx.x; t < n_tasks && !abort_s; t += gridDim.x, ++lt) {
-      const int n = tile_n(t);
-      // the epilogue has read the previous tile's accumulators
-      if (!ptx::mbar_wait(ptx::smem_u32(&acce_bar), ((uint32_t)lt & 1u) ^ 1u, deadline)) {
-        atomicOr(err, DEV_ERR_TIMEOUT_ACCUM);
-        abort_s = 1;
-        break;
-      }
-      ptx::tc_fence_after();
-      for (int i = 0; i < nkb; ++i) {
-        if (!ptx::mbar_wait(ptx::smem_u32(&full_bar[st]), ph, deadline)) {
-          atomicOr(err, DEV_ERR_TIMEOUT_FULL);
-          abort_s = 1;
-          break;
-        }
-        ptx::tc_fence_after();
-        const uint32_t sa = ptx::smem_u32(smem + (size_t)st * kDwStage);
-        const uint64_t da = ptx::sw128_desc(sa), db = ptx::sw128_desc(sa + A_BYTES);
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk)
-          ptx::mma_f16(tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc, (i > 0 || kk > 0) ? 1u : 0u);
-        const int j = i - n * half;  // position in this tile's dW half of K
-        if (j >= 0 && j < half) {
-          const uint64_t dv = ptx::sw128_desc(sa + A_BYTES + B_BYTES);
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            ptx::mma_f16(tmem + 256u, da + (uint64_t)(2 * kk), dv + (uint64_t)(2 * kk), idesc_dw,
-                         (j > 0 || kk > 0) ? 1u : 0u);
-        }
-        ptx::mma_commit(ptx::smem_u32(&empty_bar[st]));
-        if (++st == STAGES) {
-          st = 0;
-          ph ^= 1u;
-        }
-      }
-      if (abort_s) break;
-      ptx::mma_commit(ptx::smem_u32(&accf_bar));
-    }
-    if (abort_s) {
-      ptx::mma_commit(ptx::smem_u32(&drain_bar));
-      if (!ptx::mbar_wait(ptx::smem_u32(&drain_bar), 0u, ptx::drain_deadline(timeout_ns)))
-        atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
-    }
-  } else if (warp >= 2) {
-    // ---------------- epilogue ----------------
-    const int grp = warp & 3;           // TMEM lanes 32 grp .. 32 grp + 31
-    const int third = (warp - 2) >> 2;  // DFT column chunks third, third + 3, ...; third 0 also takes dW
-    int lt = 0;
-    for (int t = blockIdx.x; t < n_tasks; t += gridDim.x, ++lt) {
-      const int m0 = tile_m0(t), n = tile_n(t);
-      bool ok = true;
-      for (;;) {
-        if (ptx::mbar_try_wait(ptx::smem_u32(&accf_bar), (uint32_t)lt & 1u)) break;
-        if (abort_s || ptx::globaltimer() > deadline) {
-          ok = false;
-          break;
-        }
-      }
-      if (!__all_sync(0xffffffffu, ok)) {
-        if (lane == 0 && !abort_s) atomicOr(err, DEV_ERR_TIMEOUT_ACCUM);
-        abort_s = 1;
-        break;
-      }
-      ptx::tc_fence_after();
-      const int row = m0 + grp * 32 + lane;
-      const uint32_t lane_addr = tmem + ((uint32_t)(grp * 32) << 16);
-      auto load32 = [&](uint32_t col, float (&a)[32]) {
-        uint32_t r0[8], r1[8], r2[8], r3[8];
-        ptx::tmem_ld_x8(lane_addr + col, r0);
-        ptx::tmem_ld_x8(lane_addr + col + 8u, r1);
-        ptx::tmem_ld_x8(lane_addr + col + 16u, r2);
-        ptx::tmem_ld_x8(lane_addr + col + 24u, r3);
-        ptx::tmem_wait_ld();
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          a[q] = __uint_as_float(r0[q]);
-          a[8 + q] = __uint_as_float(r1[q]);
-          a[16 + q] = __uint_as_float(r2[q]);
-          a[24 + q] = __uint_as_float(r3[q]);
-        }
-      };
-#pragma unroll 1
-      for (int c = third; c < BN / 32; c += 3) {
-        if (n * BN + 32 * c >= ea.cols) break;  // warp-uniform
-        float a[32];
-        load32((uint32_t)(32 * c), a);
-        epilogue<EPI_MODES, __nv_bfloat16, true>(ea, nullptr, nullptr, row, n * BN + 32 * c, 0, a);
-      }
-      if (third == 0) {  // the diagonal block of this quadrant's sample: dW_b partial, K half n
-        float a[32];
-        load32(256u + (uint32_t)(32 * grp), a);
-        epilogue<EPI_DW, __nv_bfloat16, true>(ew, nullptr, nullptr, row, 32 * grp, n, a);
-      }
-      ptx::tc_fence_before();
-      __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&acce_bar));
-    }
-  }
-
-  // ---------------- teardown ----------------
-  __syncwarp();
-  ptx::tc_fence_before();
-  __syncthreads();
-  if (warp == 0) {
-    ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem, 512);
-  }
-}
-
-cudaError_t launch_gemm_dft_dw(const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mV,
-                               const EpiArgs& ea, const EpiArgs& ew, int M, int N, int K, int* err,
-                               uint64_t timeout_ns, cudaStream_t st) {
-  if (N != 512 || K % 128 != 0 || ew.splits != 2) return cudaErrorInvalidValue;
-  const void* fn = reinterpret_cast<const void*>(gemm_dft_dw_kernel);
-  cudaError_t e = allow_max_smem(fn);
-  if (e != cudaSuccess) return e;
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int m_tiles = (M + 127) / 128;
-  const int grid = std::max(1, std::min(2 * m_tiles, sms));
-  gemm_dft_dw_kernel<<<grid, kLayerThreads, kDwSmem, st>>>(mA, mB, mV, ea, ew, K, m_tiles, err, timeout_ns);
   return cudaGetLastError();
 }
 
@@ -858,18 +631,10 @@ cudaError_t launch_gemm_tc(int epi, int BN, const CUtensorMap& mA, const CUtenso
   // the 1x1 segment shares the accumulator: the DFT part must come pre-scaled (alpha 1)
   if (layer && (splits != 1 || BN != 256 || ea.alpha != 1.0f)) return cudaErrorInvalidValue;
   switch (epi) {
-    case EPI_MODES:
-      // BN 256 without K splits: the persistent form (four stages, overlapped epilogue)
-      if (BN == 256 && splits == 1)
-        return launch_layer_persistent<EPI_MODES>(mA, mB, mA2, mW, ea, M, N, K, err, timeout_ns, st);
-      return launch_tc_bn<EPI_MODES>(BN, mA, mB, mA2, mW, ea, M, N, K, splits, err, timeout_ns, st);
     case EPI_LAYER_FWD:
       return launch_layer_persistent<EPI_LAYER_FWD>(mA, mB, mA2, mW, ea, M, N, K, err, timeout_ns, st);
     case EPI_LAYER_BWD:
       return launch_layer_persistent<EPI_LAYER_BWD>(mA, mB, mA2, mW, ea, M, N, K, err, timeout_ns, st);
-    case EPI_DW:
-      return BN == 128 ? launch_tc_t<128, EPI_DW>(mA, mB, mA2, mW, ea, M, N, K, splits, err, timeout_ns, st)
-                       : cudaErrorInvalidValue;
     case EPI_FIELD:
       if (splits != 1) return cudaErrorInvalidValue;
       // BN 256: the persistent form (epilogue of one tile overlapping the next tile's MMAs)
@@ -877,14 +642,6 @@ cudaError_t launch_gemm_tc(int epi, int BN, const CUtensorMap& mA, const CUtenso
                        : launch_tc_bn<EPI_FIELD>(BN, mA, mB, mA2, mW, ea, M, N, K, 1, err, timeout_ns, st);
     default: return cudaErrorInvalidValue;
   }
-}
-
-int gemm_tc_ctas_per_sm(int BN) {
-  const uint32_t smem = BN == 32    ? GemmCfg<32>::SMEM
-                        : BN == 64  ? GemmCfg<64>::SMEM
-                        : BN == 128 ? GemmCfg<128>::SMEM
-                                    : GemmCfg<256>::SMEM;
-  return smem <= 110u * 1024u ? 2 : 1;
 }
 
 template <int EPI>

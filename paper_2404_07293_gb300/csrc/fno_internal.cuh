@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <vector>
 
 #include "scw_internal.cuh"
 
@@ -20,8 +21,8 @@ constexpr int PIX_BLOCK = 256;  // pixels per block of the per-pixel kernels (N*
 
 // GEMM epilogues. Rows / columns are those of the GEMM's D = A B^T.
 enum Epi : int {
-  EPI_MODES = 0,      // rows = (sample, channel), columns = (mode, re/im): alpha D -> mode-major complex
-                      // out[split][mode][row] (truncated DFTs)
+  EPI_MODES = 0,      // rows = (sample, channel), columns = (independent mode, re/im): alpha D and its
+                      // conjugate partner -> mode-major complex out[split][mode][row] (truncated DFTs)
   EPI_LAYER_FWD = 1,  // rows = pixels, columns = (sample, channel): Z = alpha D + c + W V; V' = GELU(Z)
   EPI_LAYER_BWD = 2,  // rows = pixels, columns = (sample, channel): dV = D + W^T dZ; dZ' = dV GELU'(Z)
                       // (GELU'(Z) stored by the forward)
@@ -51,6 +52,8 @@ struct EpiArgs {
   int gelu;            // FWD: apply GELU
   int fz_out;          // FIELD: output planes per illumination
   int illum;           // FIELD: illuminations I
+  const int2* modes;   // EPI_MODES: columns 2j, 2j + 1 are the independent mode j; modes[j] = (its mode index,
+                       // the index of its conjugate partner or -1)
 };
 
 // ---- element access (T = float or __nv_bfloat16) ----------------------------------------
@@ -191,7 +194,12 @@ __device__ __forceinline__ void epilogue(const EpiArgs& a, const float* w_s, con
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       const int k = col0 / 2 + j;
-      if (2 * k < a.cols) o[(size_t)k * a.ld] = make_float2(a.alpha * acc[2 * j], a.alpha * acc[2 * j + 1]);
+      if (2 * k < a.cols) {
+        const int2 md = a.modes[k];
+        const float2 v = make_float2(a.alpha * acc[2 * j], a.alpha * acc[2 * j + 1]);
+        o[(size_t)md.x * a.ld] = v;
+        if (md.y >= 0) o[(size_t)md.y * a.ld] = make_float2(v.x, -v.y);
+      }
     }
   } else if constexpr (EPI == EPI_FIELD) {
     if (row >= a.rows) return;
@@ -301,8 +309,7 @@ __device__ __forceinline__ void epilogue(const EpiArgs& a, const float* w_s, con
 // ---- launchers ---------------------------------------------------------------------------
 // Tensor-core GEMM D = A B^T over K (bf16, K-major, TMA maps with 128-byte swizzle and
 // a 64-element inner box): A rows in boxes of 128, B rows in boxes of BN (32..256).
-// grid = (ceil(M/128), ceil(N/BN), splits); EPI_DW uses grid.x = groups and the same row
-// offset for A and B. Each split covers kper 64-wide K blocks.
+// grid = (ceil(N/BN), ceil(M/128), splits). Each split covers kper 64-wide K blocks.
 // EPI_LAYER_*: mA2 / mW are the 1x1-convolution operands (channel-first activations [B][C][P]
 // as a 3D map with box {64, 32, kSeg2Samples} and 128-byte swizzle, read MN-major; W or W^T
 // [C][C] with box {32, 32} and 64-byte swizzle); they run on the tensor cores as one extra
@@ -311,18 +318,21 @@ __device__ __forceinline__ void epilogue(const EpiArgs& a, const float* w_s, con
 cudaError_t launch_gemm_tc(int epi, int BN, const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mA2,
                            const CUtensorMap& mW, const EpiArgs& ea, int M, int N, int K, int splits, int* err,
                            uint64_t timeout_ns, cudaStream_t st);
-// Backward truncated DFT of dZ (EPI_MODES into ea, N = 2 m^2 = 512 columns, two tiles of 256)
-// fused with the weight gradient (EPI_DW into ew, ew.splits = 2: the two column tiles each take one
-// half of K = pixels, a multiple of 128): mA = dZ channel-first, mB = the DFT table D, mV = V
-// channel-first (box 128 rows). Tensor-core (BF16) mode only.
-cudaError_t launch_gemm_dft_dw(const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mV,
-                               const EpiArgs& ea, const EpiArgs& ew, int M, int N, int K, int* err,
-                               uint64_t timeout_ns, cudaStream_t st);
+// Truncated DFT (EPI_MODES into ea) on the tensor cores: M = rows of A (channel-first activations, box
+// 128 rows), N = 2 x independent modes, K = pixels (a multiple of 128), mB[i] = the DFT table with boxes of
+// kDftTiles[i] rows. With ew / mV it also forms the weight gradient (EPI_DW, ew->splits = 2: the first
+// two column tiles take one half of the pixels each) from A = dZ and mV = V channel-first.
+constexpr int kDftTileCount = 5;
+constexpr int kDftTiles[kDftTileCount] = {16, 32, 48, 96, 144};
+int dft_tile(int M, int N, int sms);
+cudaError_t launch_dft_tc(const CUtensorMap& mA, const CUtensorMap* mB, const CUtensorMap* mV, const EpiArgs& ea,
+                          const EpiArgs* ew, int M, int N, int K, int* err, uint64_t timeout_ns, cudaStream_t st);
+// The modes the DFTs multiply, in the order of the table's rows: (mode index, conjugate partner or -1).
+int dft_independent_modes(int m, std::vector<int2>& modes);
 // FP32 SIMT GEMM with the same semantics (A [M][lda], B [N][ldb] row-major FP32; for EPI_DW
 // rows of B are offset like rows of A).
 cudaError_t launch_gemm_simt(int epi, const float* A, long long lda, const float* B, long long ldb,
                              const EpiArgs& ea, int M, int N, int K, int splits, cudaStream_t st);
-int gemm_tc_ctas_per_sm(int BN);
 
 // encode a 2D bf16 tensor map: `rows` rows of `cols` elements (row pitch `pitch` elements),
 // box {box_cols, box_rows} with box_cols 64 (128-byte swizzle) or 32 (64-byte swizzle),
@@ -337,7 +347,7 @@ constexpr int kSeg2Samples = 4;
 scw_status make_map_act3d(CUtensorMap* m, const void* base, long long P, long long samples);
 
 template <typename T>
-cudaError_t launch_tables(T* D, T* E, int N, int m, int Kp, cudaStream_t st);
+cudaError_t launch_tables(T* D, T* E, const int2* modes, int n_modes, int N, int m, int Kp, cudaStream_t st);
 template <typename T>
 cudaError_t launch_lift(const float2* n, const T* params, T* Vcf, T* Vcl, int B, int S, int in_grid, int N,
                         cudaStream_t st);

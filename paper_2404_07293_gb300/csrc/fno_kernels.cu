@@ -8,24 +8,28 @@
 namespace scw {
 namespace fno {
 
-// ---- DFT tables: D[2k + r][p] = cos(theta) (r = 0) or -sin(theta) (r = 1), E = D^T (pads zero)
+// ---- DFT tables: E[p][2k + r] = cos(theta) (r = 0) or -sin(theta) (r = 1) for every kept mode k (pads
+// zero), D[2j + r][p] the same for the independent modes k = modes[j].x (one of each conjugate pair).
 // theta = 2 pi ((kx x + ky y) mod N) / N, reduced exactly in integers, evaluated in FP64.
+__device__ __forceinline__ float dft_value(int k, int r, int p, int N, int m) {
+  const int ky = k / m - m / 2, kx = k % m - m / 2;
+  const int y = p / N, x = p % N;
+  const int a = (((kx * x + ky * y) % N) + N) % N;
+  double s, c;
+  sincospi(2.0 * a / N, &s, &c);
+  return r ? (float)-s : (float)c;
+}
+
 template <typename T>
-__global__ void tables_kernel(T* __restrict__ D, T* __restrict__ E, int N, int m, int Kp) {
+__global__ void tables_kernel(T* __restrict__ D, T* __restrict__ E, const int2* __restrict__ modes, int n_modes, int N,
+                              int m, int Kp) {
   const int P = N * N, Kc = 2 * m * m;
   const long long total = (long long)Kc * P;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
        idx += (long long)gridDim.x * blockDim.x) {
     const int q = (int)(idx / P), p = (int)(idx % P);
-    const int k = q >> 1;
-    const int ky = k / m - m / 2, kx = k % m - m / 2;
-    const int y = p / N, x = p % N;
-    const int r = (((kx * x + ky * y) % N) + N) % N;
-    double s, c;
-    sincospi(2.0 * r / N, &s, &c);
-    const float v = (q & 1) ? (float)-s : (float)c;
-    D[(size_t)q * P + p] = from_f<T>(v);
-    E[(size_t)p * Kp + q] = from_f<T>(v);
+    E[(size_t)p * Kp + q] = from_f<T>(dft_value(q >> 1, q & 1, p, N, m));
+    if (q < 2 * n_modes) D[(size_t)q * P + p] = from_f<T>(dft_value(modes[q >> 1].x, q & 1, p, N, m));
   }
 }
 
@@ -836,9 +840,8 @@ static int blocks_for(long long n, int threads, int cap = 152 * 16) {
 }
 
 template <typename T>
-cudaError_t launch_tables(T* D, T* E, int N, int m, int Kp, cudaStream_t st) {
-  const long long n = 2LL * m * m * N * N;
-  tables_kernel<T><<<blocks_for(n, 256), 256, 0, st>>>(D, E, N, m, Kp);
+cudaError_t launch_tables(T* D, T* E, const int2* modes, int n_modes, int N, int m, int Kp, cudaStream_t st) {
+  tables_kernel<T><<<blocks_for(2LL * m * m * N * N, 256), 256, 0, st>>>(D, E, modes, n_modes, N, m, Kp);
   return cudaGetLastError();
 }
 
@@ -1056,13 +1059,13 @@ cudaError_t launch_project_infer(const T* Vcl, const T* params_q, float2* field,
 template <typename T>
 cudaError_t launch_head_infer(const float* part_pool, const T* params_e, float q, float threshold, float* h_out,
                               float* est, unsigned char* flag, int B, int P, cudaStream_t st) {
-  head_infer_kernel<T><<<(B + 127) / 128, 128, 0, st>>>(part_pool, params_e, q, threshold, h_out, est, flag, B,
+  head_infer_kernel<T><<<(B + 3) / 4, 128, 0, st>>>(part_pool, params_e, q, threshold, h_out, est, flag, B,
                                                         P / PIX_BLOCK, P);
   return cudaGetLastError();
 }
 
 #define SCW_FNO_INSTANTIATE(T)                                                                                       \
-  template cudaError_t launch_tables<T>(T*, T*, int, int, int, cudaStream_t);                                      \
+  template cudaError_t launch_tables<T>(T*, T*, const int2*, int, int, int, int, cudaStream_t);                                      \
   template cudaError_t launch_lift<T>(const float2*, const T*, T*, T*, int, int, int, int, cudaStream_t);          \
   template cudaError_t launch_mix_fwd<T>(const float2*, int, long long, long long, const T*, T*, float, int, int, \
                                          int, cudaStream_t);                                                        \
