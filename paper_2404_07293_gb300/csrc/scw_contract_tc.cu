@@ -12,15 +12,16 @@
 // Persistent, warp-specialised kernel. Work is a list of tasks (item, unit,
 // 128-row tile, K split), grouped per CTA on the host longest-first; every role
 // walks the same list:
-//   warp 0 lane 0   producer: contiguous cp.async.bulk copies (no multicast) of
+//   warp 0          producer: contiguous cp.async.bulk copies (no multicast) of
 //                   the pre-swizzled tile-major A tiles (L2 evict-first: W is
 //                   streamed once) and B chunks (evict-last: re-read by every row
 //                   tile) into a ring of shared-memory stages (full/empty mbarriers)
-//   warp 1 lane 0   tcgen05.mma issuer (M = 128, N = NB, K = 16 per instruction)
+//   warp 1          tcgen05.mma issuer (M = 128, N = NB, K = 16 per instruction)
 //                   into one of two TMEM accumulators (acc_full/acc_empty)
 //   warps 2-5       epilogue: tcgen05.ld 32 lanes x 8 columns of the other
 //                   accumulator, coalesced stores of S_part[split][plane][row]
-// so loads, MMAs and the previous task's epilogue overlap. Every wait is bounded
+// so loads, MMAs and the previous task's epilogue overlap. Both issuing roles run warp-converged with
+// one elected lane (ptx::elect_one). Every wait is bounded
 // by a %globaltimer deadline; a timeout sets the error word and all roles stop.
 #include "scw_internal.cuh"
 #include "scw_ptx.cuh"
@@ -111,8 +112,9 @@ __global__ void __launch_bounds__(192) contract_tc_kernel(const __grid_constant_
   ptx::tc_fence_after();
   const uint32_t tmem = tmem_base_s;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ---------------- bulk-copy producer ----------------
+    const uint32_t leader = ptx::elect_one();
     const uint64_t pol_a = ptx::policy_evict_first(), pol_b = ptx::policy_evict_last();
     int st = 0;
     uint32_t ph = 0;
@@ -127,13 +129,13 @@ __global__ void __launch_bounds__(192) contract_tc_kernel(const __grid_constant_
     auto flush_pending = [&]() {
       ptx::griddep_wait();
       for (int q = 0; q < npend; ++q) {
-        ptx::bulk_load(pend_sb[q], pend_bh[q], Cfg::B_BYTES, pend_fb[q], pol_b);
-        ptx::bulk_load(pend_sb[q] + Cfg::B_BYTES, pend_bl[q], Cfg::B_BYTES, pend_fb[q], pol_b);
+        ptx::bulk_load(pend_sb[q], pend_bh[q], Cfg::B_BYTES, pend_fb[q], pol_b, leader);
+        ptx::bulk_load(pend_sb[q] + Cfg::B_BYTES, pend_bl[q], Cfg::B_BYTES, pend_fb[q], pol_b, leader);
       }
       npend = 0;
       dep_done = true;
     };
-    for (int t = t_begin; t < t_end && !abort_s; ++t) {
+    for (int t = t_begin; t < t_end && !ptx::warp_any(abort_s); ++t) {
       const int4 tk = tasks[t];
       const ItemDev& it = BATCH ? items[tk.x] : one;
       const TaskGeom g = task_geom(tk, it);
@@ -148,8 +150,8 @@ __global__ void __launch_bounds__(192) contract_tc_kernel(const __grid_constant_
       const uint16_t* Bh = static_cast<const uint16_t*>(it.Bhi);
       const uint16_t* Bl = static_cast<const uint16_t*>(it.Blo);
       for (int i = 0; i < g.kcount; ++i) {
-        if (!ptx::mbar_wait(ptx::smem_u32(&empty_bar[st]), ph ^ 1u, deadline)) {
-          atomicOr(err, DEV_ERR_TIMEOUT_EMPTY);
+        if (!ptx::mbar_wait_warp(ptx::smem_u32(&empty_bar[st]), ph ^ 1u, deadline)) {
+          if (leader) atomicOr(err, DEV_ERR_TIMEOUT_EMPTY);
           abort_s = 1;
           break;
         }
@@ -157,17 +159,17 @@ __global__ void __launch_bounds__(192) contract_tc_kernel(const __grid_constant_
         if (inject_stall && blockIdx.x == 0 && issued == 0) {
           skipped = 0;  // failure injection (scw_plan_inject_stall): this stage is never filled
         } else {
-          ptx::mbar_arrive_expect_tx(fb, tx);
+          ptx::mbar_arrive_expect_tx(fb, tx, leader);
           const int kc = g.kb + i;
           const uint32_t sa = ptx::smem_u32(smem + (size_t)st * Cfg::STAGE_BYTES);
           const size_t ao = a0 + (size_t)kc * g.rt * 64;
-          ptx::bulk_load(sa, Ah + ao, a_bytes, fb, pol_a);
-          if (SPLIT) ptx::bulk_load(sa + Cfg::A_BYTES, Al + ao, a_bytes, fb, pol_a);
+          ptx::bulk_load(sa, Ah + ao, a_bytes, fb, pol_a, leader);
+          if (SPLIT) ptx::bulk_load(sa + Cfg::A_BYTES, Al + ao, a_bytes, fb, pol_a, leader);
           const uint32_t sb = sa + Cfg::NA * Cfg::A_BYTES;
           const size_t bo = b0 + (size_t)kc * NB * 64;
           if (dep_done) {
-            ptx::bulk_load(sb, Bh + bo, Cfg::B_BYTES, fb, pol_b);
-            ptx::bulk_load(sb + Cfg::B_BYTES, Bl + bo, Cfg::B_BYTES, fb, pol_b);
+            ptx::bulk_load(sb, Bh + bo, Cfg::B_BYTES, fb, pol_b, leader);
+            ptx::bulk_load(sb + Cfg::B_BYTES, Bl + bo, Cfg::B_BYTES, fb, pol_b, leader);
           } else {
             pend_sb[npend] = sb;
             pend_fb[npend] = fb;
@@ -184,39 +186,40 @@ __global__ void __launch_bounds__(192) contract_tc_kernel(const __grid_constant_
       }
     }
     if (!dep_done) flush_pending();  // fewer stages than the ring, or an early stop
-    if (abort_s) {
+    if (ptx::warp_any(abort_s)) {
       // let the last issued copies land before the CTA's shared memory goes away
       const uint64_t d2 = ptx::drain_deadline(timeout_ns);
       for (int back = 1; back <= STAGES && back <= issued; ++back) {
         const int i = issued - back;
         if (i == skipped) continue;  // nothing was sent to that stage
-        if (!ptx::mbar_wait(ptx::smem_u32(&full_bar[i % STAGES]), (uint32_t)(i / STAGES) & 1u, d2)) {
-          atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
+        if (!ptx::mbar_wait_warp(ptx::smem_u32(&full_bar[i % STAGES]), (uint32_t)(i / STAGES) & 1u, d2)) {
+          if (leader) atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
           break;
         }
       }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------- tcgen05.mma issuer ----------------
+    const uint32_t leader = ptx::elect_one();
     constexpr uint32_t idesc = ptx::idesc_f16(SPLIT, 128, NB);
     int st = 0;
     uint32_t ph = 0;
     int lt = 0;
-    for (int t = t_begin; t < t_end && !abort_s; ++t, ++lt) {
+    for (int t = t_begin; t < t_end && !ptx::warp_any(abort_s); ++t, ++lt) {
       const int4 tk = tasks[t];
       const ItemDev& it = BATCH ? items[tk.x] : one;
       const TaskGeom g = task_geom(tk, it);
       const int acc = lt & 1;
-      if (!ptx::mbar_wait(ptx::smem_u32(&acce_bar[acc]), ((uint32_t)(lt >> 1) & 1u) ^ 1u, deadline)) {
-        atomicOr(err, DEV_ERR_TIMEOUT_ACCUM);
+      if (!ptx::mbar_wait_warp(ptx::smem_u32(&acce_bar[acc]), ((uint32_t)(lt >> 1) & 1u) ^ 1u, deadline)) {
+        if (leader) atomicOr(err, DEV_ERR_TIMEOUT_ACCUM);
         abort_s = 1;
         break;
       }
       ptx::tc_fence_after();
       const uint32_t d_tmem = tmem + (uint32_t)acc * Cfg::ACC_COLS;
       for (int i = 0; i < g.kcount; ++i) {
-        if (!ptx::mbar_wait(ptx::smem_u32(&full_bar[st]), ph, deadline)) {
-          atomicOr(err, DEV_ERR_TIMEOUT_FULL);
+        if (!ptx::mbar_wait_warp(ptx::smem_u32(&full_bar[st]), ph, deadline)) {
+          if (leader) atomicOr(err, DEV_ERR_TIMEOUT_FULL);
           abort_s = 1;
           break;
         }
@@ -231,23 +234,23 @@ __global__ void __launch_bounds__(192) contract_tc_kernel(const __grid_constant_
         for (int kk = 0; kk < 4; ++kk) {
           // K advance of 16 elements = 32 bytes inside the 128-byte swizzle row
           const uint64_t o = (uint64_t)(2 * kk);
-          ptx::mma_f16(d_tmem, dah + o, dbh + o, idesc, (i > 0 || kk > 0) ? 1u : 0u);
-          ptx::mma_f16(d_tmem, dah + o, dbl + o, idesc, 1u);
-          if (SPLIT) ptx::mma_f16(d_tmem, dal + o, dbh + o, idesc, 1u);
+          ptx::mma_f16(d_tmem, dah + o, dbh + o, idesc, (i > 0 || kk > 0) ? 1u : 0u, leader);
+          ptx::mma_f16(d_tmem, dah + o, dbl + o, idesc, 1u, leader);
+          if (SPLIT) ptx::mma_f16(d_tmem, dal + o, dbh + o, idesc, 1u, leader);
         }
-        ptx::mma_commit(ptx::smem_u32(&empty_bar[st]));
+        ptx::mma_commit(ptx::smem_u32(&empty_bar[st]), leader);
         if (++st == STAGES) {
           st = 0;
           ph ^= 1u;
         }
       }
-      ptx::mma_commit(ptx::smem_u32(&accf_bar[acc]));
+      ptx::mma_commit(ptx::smem_u32(&accf_bar[acc]), leader);
     }
-    if (abort_s) {
+    if (ptx::warp_any(abort_s)) {
       // issued MMAs must finish before the tensor memory is released
-      ptx::mma_commit(ptx::smem_u32(&drain_bar));
-      if (!ptx::mbar_wait(ptx::smem_u32(&drain_bar), 0u, ptx::drain_deadline(timeout_ns)))
-        atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
+      ptx::mma_commit(ptx::smem_u32(&drain_bar), leader);
+      if (!ptx::mbar_wait_warp(ptx::smem_u32(&drain_bar), 0u, ptx::drain_deadline(timeout_ns)))
+        if (leader) atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
     }
   } else if (warp >= 2) {
     // ---------------- epilogue ----------------
