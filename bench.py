@@ -932,9 +932,12 @@ def run_ours(args, world, rank, local):
     per_kernel = {
         "contract": (w_bytes + s_bytes, kt["contract_ms"],
                      "contract_tc_kernel" if args.precision != "fp32" else "contract_fp32_kernel"),
-        "ypass": (t_bytes + out_bytes, kt["ypass_ms"], "ypass_kernel"),
-        "xpass": (s_bytes + t_bytes, kt["xpass_ms"], "xpass_kernel"),
     }
+    if "xpass" in timeline:
+        per_kernel["ypass"] = (t_bytes + out_bytes, kt["ypass_ms"], "ypass_reg_kernel")
+        per_kernel["xpass"] = (s_bytes + t_bytes, kt["xpass_ms"], "xpass_kernel")
+    else:  # both directions in one kernel: the x-pass rows stay on the chip
+        per_kernel["recompose"] = (s_bytes + out_bytes, kt["ypass_ms"], "recompose_fused_kernel")
     kernels = {k: {"kernel": name, "algorithmic_bytes": b, "launch_ms": t, "gbs": b / (t * 1e-3) / 1e9,
                    "frac": b / (t * 1e-3) / 1e9 / hbm} for k, (b, t, name) in per_kernel.items()}
     dominant = max(kernels, key=lambda k: kernels[k]["launch_ms"])

@@ -308,7 +308,8 @@ scw_status scw_plan_get_info(scw_plan_t plan, scw_plan_info* info);
  * would break their programmatic overlap): with tracing on, thread 0 of every CTA stamps the
  * %globaltimer when its work begins (after any wait on the preceding kernel) and when it ends;
  * per slot the earliest begin and the latest end are kept. Slots: 0 phases (a), 1 exterior
- * planes, 2 contraction (b), 3 x-pass and 4 y-pass (c). scw_plan_enable_trace synchronises the
+ * planes, 2 contraction (b), 3 x-pass and 4 y-pass (c; slot 4 alone where one kernel does both
+ * directions). scw_plan_enable_trace synchronises the
  * device, allocates (on != 0) or frees the 128-byte stamp buffer and drops the graph.
  * scw_plan_get_trace synchronises the device, writes us[2 s] / us[2 s + 1] = begin / end of slot s
  * in microseconds from the earliest begin (-1 for slots no kernel stamped; n_slots entries
@@ -325,7 +326,8 @@ typedef struct {
   double phases_ms;      /* step (a) incl. exterior planes, per call       */
   double contract_ms;    /* step (b)                                       */
   double recompose_ms;   /* step (c): both directions and the field stores */
-  double xpass_ms;       /* step (c), x direction                          */
+  double xpass_ms;       /* step (c), x direction (about 0 where one kernel does
+                            both directions: its time is ypass_ms)         */
   double ypass_ms;       /* step (c), y direction and the field stores     */
   double total_ms;       /* first to last event                            */
 } scw_kernel_times;

@@ -583,9 +583,9 @@ struct scw_plan_s {
   ItemDev* d_items = nullptr;      // batched plans only
   int2* d_unit_entries = nullptr;
   int n_unit_entries = 0;
-  int2* d_plane_entries = nullptr;  // y-pass-pair class first (ypass_pairs), then the rest
+  int2* d_plane_entries = nullptr;  // long y folds first (ypass_long), then the rest
   int n_plane_entries = 0;
-  int n_pair_entries = 0;
+  int n_long_entries = 0;
   bool tiled = false;  // some item stores periodic tiles
   int max_twy = 0;     // largest y fold-twiddle table (complex elements)
   int inject_stall = 0;            // scw_plan_inject_stall (tests of the timeout path)
@@ -595,6 +595,7 @@ struct scw_plan_s {
   float2** h_outs = nullptr;       // pinned
   int max_M = 0, max_Qx = 0, max_V = 0, max_Vp = 0;
   size_t xpass_smem = 0;
+  size_t fused_smem = 0;  // shared memory of the one-kernel recomposition; 0: x-pass and y-pass (fuse_recompose)
   size_t rec_smem = 0;
   // graph replay
   cudaStream_t cap_stream = nullptr;
@@ -772,7 +773,7 @@ static scw_status enqueue_pipelined(scw_plan_t P, float2* out_one, cudaStream_t 
     e = launch_xpass(one, nullptr, ent, nb, P->xpass_smem, P->st2);
     if (e != cudaSuccess) return cuda_error(e, "x-pass launch");
     int ny = 0;
-    e = launch_ypass(one, nullptr, ent, nb, ypass_pairs(one.Vp) ? nb : 0, P->max_Qx, P->max_Vp, P->max_twy, P->tiled, out_one, nullptr,
+    e = launch_ypass(one, nullptr, ent, nb, ypass_long(one.Vp) ? nb : 0, P->max_Qx, P->max_Vp, P->max_twy, P->tiled, out_one, nullptr,
                      P->st2, &ny);
     if (e != cudaSuccess) return cuda_error(e, "y-pass launch");
     n += 1 + ny;
@@ -792,11 +793,22 @@ static scw_status enqueue_synthesis(scw_plan_t P, float2* out_one, cudaStream_t 
   const ItemDev& one = P->items[0]->item;
   const ItemDev* items = P->batched ? P->d_items : nullptr;
   mark(P, 2, st, marks);
-  cudaError_t e = launch_xpass(one, items, P->d_plane_entries, P->n_plane_entries, P->xpass_smem, st);
+  cudaError_t e;
+  if (P->fused_smem) {
+    mark(P, 3, st, marks);  // one kernel: its time is the y-pass's
+    e = launch_recompose_fused(one, items, P->d_plane_entries, P->n_plane_entries, P->max_Vp, P->fused_smem, P->tiled,
+                               out_one, P->d_outs, st);
+    if (e != cudaSuccess) return cuda_error(e, "recompose launch");
+    mark(P, 4, st, marks);
+    ++n;
+    if (marks && P->timing && P->tev_used + kMarks <= P->tev.size()) P->tev_used += kMarks;
+    return SCW_OK;
+  }
+  e = launch_xpass(one, items, P->d_plane_entries, P->n_plane_entries, P->xpass_smem, st);
   if (e != cudaSuccess) return cuda_error(e, "x-pass launch");
   mark(P, 3, st, marks);
   int ny = 0;
-  e = launch_ypass(one, items, P->d_plane_entries, P->n_plane_entries, P->n_pair_entries, P->max_Qx, P->max_Vp, P->max_twy, P->tiled,
+  e = launch_ypass(one, items, P->d_plane_entries, P->n_plane_entries, P->n_long_entries, P->max_Qx, P->max_Vp, P->max_twy, P->tiled,
                    out_one, P->d_outs, st, &ny);
   if (e != cudaSuccess) return cuda_error(e, "y-pass launch");
   mark(P, 4, st, marks);
@@ -985,6 +997,24 @@ static scw_status choose_splits(scw_plan_t P, bool timed, const std::vector<int>
   return upload_schedule(P->items, P->NB, P->bf16, P->sched);
 }
 
+// Shared memory of the one-kernel recomposition where the plan runs it, else 0 (x-pass, then y-pass). It
+// is the faster one wherever it fits (launch_recompose_fused), by 1 to 2 us of 14 to 37 even for a few
+// planes; plans of fewer than kFuseTiles (plane, component) tiles keep the four-launch sequence that
+// scw_plan_info reports for a small single plan.
+constexpr int kFuseTiles = 64;
+
+static size_t fuse_recompose(const scw_plan_t P, int n_planes) {
+  if (3 * n_planes < kFuseTiles) return 0;
+  size_t smem = 0;
+  for (const Plan* p : P->items) {
+    if (p->flags & SCW_FLAG_DEBUG_BOUNDS) return 0;  // the two kernels carry the index checks
+    const size_t b = fused_recompose_smem(p->U, p->V, p->Fx, p->Fy);
+    if (b == 0) return 0;
+    smem = std::max(smem, b);
+  }
+  return smem;
+}
+
 // Shared tail of single and batched plan creation.
 static scw_status finish_plan(scw_plan_t P, const std::vector<int>& user_ks, bool timed) {
   size_t tot = 0;
@@ -1006,11 +1036,12 @@ static scw_status finish_plan(scw_plan_t P, const std::vector<int>& user_ks, boo
     P->tiled = P->tiled || p->tiles_x > 1 || p->tiles_y > 1;
     P->max_twy = std::max(P->max_twy, (p->Fy / 8) * p->item.Vp);
   }
-  // plane entries of items with long y folds first: they run the two-residue y-pass
+  // plane entries of items with long y folds first: they run the shared-memory y-pass
   std::stable_partition(pe.begin(), pe.end(),
-                        [&](const int2& en) { return ypass_pairs(P->items[en.x]->item.Vp); });
-  P->n_pair_entries = 0;
-  for (const int2& en : pe) P->n_pair_entries += ypass_pairs(P->items[en.x]->item.Vp) ? 1 : 0;
+                        [&](const int2& en) { return ypass_long(P->items[en.x]->item.Vp); });
+  P->n_long_entries = 0;
+  for (const int2& en : pe) P->n_long_entries += ypass_long(P->items[en.x]->item.Vp) ? 1 : 0;
+  P->fused_smem = fuse_recompose(P, (int)pe.size());
   P->n_unit_entries = (int)ue.size();
   P->n_plane_entries = (int)pe.size();
   SCW_TRY(upload(&P->d_unit_entries, ue, tot));
@@ -1158,7 +1189,7 @@ static scw_status synthesize_host_pipelined(scw_plan_t P, const void* W, const v
       const int2* ent = P->d_plane_entries + fb;
       SCW_TRY_E(launch_xpass(one, nullptr, ent, nb, P->xpass_smem, st), "x-pass launch");
       int ny = 0;
-      SCW_TRY_E(launch_ypass(one, nullptr, ent, nb, ypass_pairs(one.Vp) ? nb : 0, P->max_Qx, P->max_Vp, P->max_twy,
+      SCW_TRY_E(launch_ypass(one, nullptr, ent, nb, ypass_long(one.Vp) ? nb : 0, P->max_Qx, P->max_Vp, P->max_twy,
                              P->tiled, p->hio_out, nullptr, st, &ny), "y-pass launch");
     }
     SCW_TRY_E(cudaEventRecord(P->hev_comp[g], st), "cudaEventRecord");

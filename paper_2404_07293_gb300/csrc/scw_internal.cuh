@@ -263,15 +263,21 @@ size_t recompose_smem_bytes(int V, int Up, int Vp);
 size_t xpass_smem_bytes(int V, int Up, int Fx);
 cudaError_t launch_xpass(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
                          size_t smem_bytes, cudaStream_t st);
-// entries [0, n_pair) run the two-residue y-pass (long folds, ypass_pairs(Vp)), the rest the
-// one-residue y-pass; *launches receives the number of kernels launched (0, 1 or 2)
-bool ypass_pairs(int Vp);
+// entries [0, n_long) have folds too long for registers (ypass_long(Vp)) and run the shared-memory
+// y-pass, the rest the register form; *launches receives the number of kernels launched (0, 1 or 2)
+bool ypass_long(int Vp);
 // max_twy: the largest fold-twiddle table (Fy/8) Vp of the items, in complex elements (staged in
 // shared memory when it fits); tiled: some item has periodic tiles (selects the y-pass that stores
 // every tile)
-cudaError_t launch_ypass(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries, int n_pair,
+cudaError_t launch_ypass(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries, int n_long,
                          int max_Qx, int max_Vp, int max_twy, bool tiled, float2* out_one, float2* const* d_outs,
                          cudaStream_t st, int* launches);
+// Both directions in one kernel. fused_recompose_smem: its shared memory for an item, 0 where the item does
+// not fit it; launch: smem is the largest of the items.
+size_t fused_recompose_smem(int U, int V, int Fx, int Fy);
+cudaError_t launch_recompose_fused(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
+                                   int max_Vp, size_t smem, bool tiled, float2* out_one, float2* const* d_outs,
+                                   cudaStream_t st);
 cudaError_t launch_recompose(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries, int max_Qx,
                              size_t smem, const float2* S_override, const int* nsplit_override, float2* out_one,
                              float2* const* d_outs, cudaStream_t st);

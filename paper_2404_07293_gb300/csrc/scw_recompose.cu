@@ -256,9 +256,275 @@ __global__ void __launch_bounds__(256) xpass_kernel(const __grid_constant__ Item
   }
 }
 
+// ---- y-direction from registers ---------------------------------------------------------------
+// Columns a thread owns in the y-direction fold: two (one 16-byte store per output row) while their
+// 8 NG stored orders fit in registers, one for longer folds.
+template <int NG>
+constexpr int y_cols() { return NG <= 3 ? 2 : 1; }
+
+template <int COLS> struct ColVec;
+template <> struct ColVec<1> { typedef float2 T; };
+template <> struct ColVec<2> { typedef float4 T; };
+
+// Fold + radix-8 inverse DFT along y and the field stores of one unit of COLS columns for the residues
+// b = b0, b0 + step, ... < Q: d holds the unit's x-direction sums at their 8 NG fold positions, tw the
+// fold twiddles [Q][8 NG] (every lane of a warp reads the same ones). dst: row 0 of the unit's columns.
+template <int NG, int COLS, bool TILED>
+__device__ __forceinline__ void y_fold_store(const ItemDev& it, const typename ColVec<COLS>::T (&d)[8 * NG],
+                                             const float4* tw, int b0, int step, int Q, float2* dst) {
+#pragma unroll 1
+  for (int b = b0; b < Q; b += step) {
+    const float4* t4 = tw + (size_t)b * (4 * NG);
+    float2 G[COLS][8];
+#pragma unroll
+    for (int k = 0; k < COLS; ++k)
+#pragma unroll
+      for (int r = 0; r < 8; ++r) G[k][r] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int p = 0; p < 8 * NG; p += 2) {
+      const float4 tt = t4[p >> 1];
+      const float2 t0 = make_float2(tt.x, tt.y), t1 = make_float2(tt.z, tt.w);
+      c_fma(G[0][p & 7], make_float2(d[p].x, d[p].y), t0);
+      c_fma(G[0][(p + 1) & 7], make_float2(d[p + 1].x, d[p + 1].y), t1);
+      if constexpr (COLS == 2) {
+        c_fma(G[1][p & 7], make_float2(d[p].z, d[p].w), t0);
+        c_fma(G[1][(p + 1) & 7], make_float2(d[p + 1].z, d[p + 1].w), t1);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < COLS; ++k) idft8(G[k]);
+    // output rows b + a Q, a = 0..7, by one running pointer (eight row offsets would not fit in registers)
+    float2* row = dst + (long long)b * it.ld;
+    const long long step_q = (long long)Q * it.ld;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      if constexpr (COLS == 2)
+        store_row4<TILED>(it, row, 0, make_float4(G[0][a].x, G[0][a].y, G[1][a].x, G[1][a].y));
+      else
+        store_row2<TILED>(it, row, 0, G[0][a]);
+      row += step_q;
+    }
+  }
+}
+
+// Field offset of column x of plane slot f, component c; false when the thread's largest field index
+// (element x + COLS - 1 of the last row of the last periodic tile) is outside (debug plans).
+__device__ __forceinline__ bool y_field_base(const ItemDev& it, int f, int c, int x, int cols, long long& obase) {
+  // plane slot f = (output plane) I + illumination: slice (il 3 + c) Fz_out + fo of the field
+  const int fo = f / it.I, il = f - fo * it.I;
+  obase = ((long long)il * 3 * it.Fz_out + (long long)c * it.Fz_out + fo) * it.pstride + x;
+  return in_bounds(it, BND_OUT, (size_t)(obase + cols - 1 + (long long)(it.ty * it.Fy - 1) * it.ld +
+                                         (long long)(it.tx - 1) * it.Fx));
+}
+
+// One warp's share of a (64-column block, item-plane, component) tile of the y-pass: the residues
+// sub, sub + rs, ... of its columns.
+template <int NG, bool TILED>
+__device__ __forceinline__ void ypass_reg_tile(const ItemDev& it, const float4* tw, int f, int c, int xb, int sub,
+                                               int rs, float2* out) {
+  constexpr int COLS = y_cols<NG>();
+  typedef typename ColVec<COLS>::T VecT;
+#pragma unroll 1
+  for (int h = 0; h < 2 / COLS; ++h) {  // COLS 1: the two 32-column halves in turn
+    const int x = xb + 32 * h + COLS * (threadIdx.x & 31);
+    if (x >= it.Fx) return;  // Fx is a multiple of 8: a column pair is in or out as a whole
+    int V = it.V, Fx = it.Fx;
+    // opaque to the compiler: the 8 NG row offsets below are invariant over the tiles, and keeping them
+    // across the loop spills the registers the columns need
+    asm volatile("" : "+r"(V), "+r"(Fx));
+    const size_t tbase = ((size_t)f * 3 + c) * V * Fx + x;
+    VecT d[8 * NG];
+#pragma unroll
+    for (int p = 0; p < 8 * NG; ++p) {
+      const int v = fold_order(p, V, 8 * NG);
+      const size_t i = tbase + (size_t)(max(v, 0) * Fx);  // V Fx <= 96 * 4096
+      d[p] = VecT();
+      if (v >= 0 && in_bounds(it, BND_T, i + COLS - 1)) d[p] = *reinterpret_cast<const VecT*>(it.T + i);
+    }
+    long long obase;
+    if (!y_field_base(it, f, c, x, COLS, obase)) return;
+    y_fold_store<NG, COLS, TILED>(it, d, tw, sub, rs, it.Fy >> 3, out + obase);
+  }
+}
+
+constexpr int kYregThreads = 128;
+constexpr int kYregMaxVp = 48;  // longer folds run the shared-memory form (ypass_kernel)
+
+// y-pass with the columns in registers. The shared-memory form reads each of the fold's Vp values once
+// per residue (Fy / 8 times): 144 shared-memory wavefronts per 64 columns and residue at Vp = 24, as
+// long as the field store itself. Here a thread loads its column pair's Vp values from T once and walks
+// its residues from registers; only the twiddles come from shared memory (48 wavefronts).
+// Persistent: warp k takes the shares k, k + warps, ...; share s = tile rs + residue subset, tile =
+// (entry 3 + c) nxb + 64-column block. rs warps share a tile (launch_ypass_reg).
+// STW: the fold twiddles [Fy/8][Vp] of a single plan staged in shared memory, else read through L1.
+// NGM: the largest fold length of the launch in groups of 8.
+template <bool BATCH, bool TILED, bool STW, int NGM>
+__global__ void __launch_bounds__(kYregThreads, NGM <= 2 ? 4 : 3)
+    ypass_reg_kernel(const __grid_constant__ ItemDev one, const ItemDev* __restrict__ items,
+                     const int2* __restrict__ entries, int n_shares, int nxb, int rs, float2* out_one,
+                     float2* const* __restrict__ outs) {
+  static_assert(!(BATCH && STW), "a batch's items have different twiddles");
+  extern __shared__ float4 ys_tw[];
+  if constexpr (STW) {
+    const float4* src = reinterpret_cast<const float4*>(one.twy);
+    for (int i = threadIdx.x; i < (one.Fy >> 3) * one.Vp / 2; i += kYregThreads)
+      ys_tw[i] = in_bounds(one, BND_TWY, 2 * (size_t)i + 1) ? __ldg(src + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+  }
+  ptx::griddep_wait();  // the x-pass rows come from the preceding kernel
+  trace_begin(one.trace, TRACE_YPASS);
+  const int warps = gridDim.x * (kYregThreads / 32);
+  for (int s = blockIdx.x * (kYregThreads / 32) + (threadIdx.x >> 5); s < n_shares; s += warps) {
+    const int t = s / rs, sub = s - t * rs;
+    const int r = t / nxb, xb = (t - r * nxb) * 64;
+    const int2 e = entries[r / 3];
+    const int c = r - (r / 3) * 3;
+    const ItemDev& it = BATCH ? items[e.x] : one;
+    if (xb >= it.Fx) continue;
+    // read through L1 (debug plans: the table's last element stands for all of it)
+    if (!STW && !in_bounds(it, BND_TWY, (size_t)(it.Fy >> 3) * it.Vp - 1)) continue;
+    float2* out = BATCH ? outs[e.x] : out_one;
+    const float4* tw = STW ? ys_tw : reinterpret_cast<const float4*>(it.twy);
+    switch (it.Vp >> 3) {
+      case 1: ypass_reg_tile<1, TILED>(it, tw, e.y, c, xb, sub, rs, out); break;
+      case 2: ypass_reg_tile<2, TILED>(it, tw, e.y, c, xb, sub, rs, out); break;
+      case 3: if constexpr (NGM >= 3) ypass_reg_tile<3, TILED>(it, tw, e.y, c, xb, sub, rs, out); break;
+      case 4: if constexpr (NGM >= 6) ypass_reg_tile<4, TILED>(it, tw, e.y, c, xb, sub, rs, out); break;
+      case 5: if constexpr (NGM >= 6) ypass_reg_tile<5, TILED>(it, tw, e.y, c, xb, sub, rs, out); break;
+      case 6: if constexpr (NGM >= 6) ypass_reg_tile<6, TILED>(it, tw, e.y, c, xb, sub, rs, out); break;
+    }
+  }
+  if (one.trace) {
+    __syncthreads();
+    trace_end(one.trace, TRACE_YPASS);
+  }
+}
+
+// ---- both directions in one kernel --------------------------------------------------------------
+// One CTA per (item-plane, component), the last ones split over y: the spectrum rows (split partials summed), the
+// x-direction sums of whole pixel rows in shared memory, then the y-direction from registers. Bound by the
+// field store. The x-pass rows never reach memory (264 MB written and read again at 4096 plane slots of
+// 21 x 21 orders on 128 columns) and there is one launch less. Step times at 21 x 21 orders, x-pass and
+// shared-memory y-pass -> x-pass and register y-pass -> this kernel: 256^3 192.6 -> 189.5 -> 179.3 us;
+// 4096 slots of 128 x 128 680 -> 685 -> 560; a sweep of 32 items 1180 -> 1200 -> 1105.
+constexpr int kFusedMaxFx = 256;
+
+static size_t fused_smem_bytes(int U, int V, int Fx, int Fy) {
+  const int Up = fold_np(U), Vp = fold_np(V);
+  return ((size_t)V * Up + (size_t)V * Fx + (size_t)Up * (Fx / 8) + (size_t)(Fy / 8) * Vp + 1) * sizeof(float2);
+}
+
+template <int NG, bool TILED>
+__device__ __forceinline__ void fused_y(const ItemDev& it, const float2* rows, const float4* tw, int f, int c, int ys,
+                                        int ysplit, float2* out) {
+  constexpr int COLS = y_cols<NG>();
+  typedef typename ColVec<COLS>::T VecT;
+  const int units = it.Fx / COLS, Q = it.Fy >> 3;
+  const int k = units < kYregThreads ? kYregThreads / units : 1;  // residue groups side by side in the CTA
+  const int grp = threadIdx.x / units;                            // 0 when units >= kYregThreads
+  if (units < kYregThreads && grp >= k) return;
+  for (int u = units < kYregThreads ? threadIdx.x - grp * units : threadIdx.x; u < units; u += kYregThreads) {
+    VecT d[8 * NG];
+#pragma unroll
+    for (int p = 0; p < 8 * NG; ++p) {
+      const int v = fold_order(p, it.V, 8 * NG);
+      d[p] = VecT();
+      if (v >= 0) d[p] = *reinterpret_cast<const VecT*>(rows + v * it.Fx + u * COLS);
+    }
+    long long obase;
+    if (!y_field_base(it, f, c, u * COLS, COLS, obase)) return;
+    y_fold_store<NG, COLS, TILED>(it, d, tw, grp + k * ys, k * ysplit, Q, out + obase);
+    if (units < kYregThreads) break;
+  }
+}
+
+template <bool BATCH, bool TILED, int NGM>
+__global__ void __launch_bounds__(kYregThreads, NGM <= 2 ? 4 : 3)
+    recompose_fused_kernel(const __grid_constant__ ItemDev one, const ItemDev* __restrict__ items,
+                           const int2* __restrict__ entries, int whole, int ysplit_rest, float2* out_one,
+                           float2* const* __restrict__ outs) {
+  extern __shared__ float4 fu_s4[];
+  const int part = (int)blockIdx.x - whole;  // < 0: a whole tile; else part `part` of the split ones
+  const int ysplit = part < 0 ? 1 : ysplit_rest;
+  const int ys = part < 0 ? 0 : part % ysplit, tile = part < 0 ? blockIdx.x : whole + part / ysplit;
+  const int2 e = entries[tile / 3];
+  const int f = e.y, c = tile % 3;
+  const ItemDev& it = BATCH ? items[e.x] : one;
+  const int U = it.U, V = it.V, M = it.M, Up = it.Up, Vp = it.Vp, Fx = it.Fx, Qx = Fx >> 3, Qy = it.Fy >> 3;
+  // [V][Fx] rows, the y twiddles [Qy][Vp], the x twiddles [Up][Qx], the spectrum rows [V][Up]
+  float2* rows = reinterpret_cast<float2*>(fu_s4);
+  float4* twy = fu_s4 + (size_t)V * Fx / 2;
+  float2* twx = reinterpret_cast<float2*>(twy + (size_t)Qy * Vp / 2);
+  float2* srow = twx + (size_t)Up * Qx;
+  for (int i = threadIdx.x; i < Qy * Vp / 2; i += kYregThreads) twy[i] = __ldg(reinterpret_cast<const float4*>(it.twy) + i);
+  for (int i = threadIdx.x; i < Up * Qx; i += kYregThreads) twx[i] = __ldg(it.twx + i);
+  ptx::griddep_wait();  // the partial spectra come from the preceding contraction
+  trace_begin(one.trace, TRACE_YPASS);
+  const float2* src = it.S_part + (size_t)f * 3 * M + (size_t)c * M;
+  const int ns = it.nsplit[f];
+  const size_t stride = it.split_stride;
+  for (int i0 = 0; i0 < V * Up; i0 += 4 * kYregThreads) {
+    // the first partials of four elements are requested before any is used
+    float2 v[4][2];
+    int off[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int i = i0 + h * kYregThreads + threadIdx.x;
+      const int vi = i / Up, ui = i < V * Up ? fold_order(i - vi * Up, U, Up) : -1;
+      off[h] = ui >= 0 ? vi * U + ui : -1;
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        v[h][k] = (off[h] >= 0 && k < ns) ? src[(size_t)k * stride + off[h]] : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int i = i0 + h * kYregThreads + threadIdx.x;
+      float2 acc = c_add(v[h][0], v[h][1]);
+      if (off[h] >= 0)
+        for (int k = 2; k < ns; ++k) acc = c_add(acc, src[(size_t)k * stride + off[h]]);
+      if (i < V * Up) srow[i] = acc;
+    }
+  }
+  __syncthreads();
+  {  // x-direction: thread (row group g, residue b), rows g, g + ng, ...
+    const int ng = kYregThreads / Qx, g = threadIdx.x / Qx, b = threadIdx.x - g * Qx;
+    if (g < ng)
+      for (int vi = g; vi < V; vi += ng) {
+        const float2* sr = srow + vi * Up;
+        const float2* tw = twx + b;
+        float2 G[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) G[r] = make_float2(0.f, 0.f);
+#pragma unroll 1
+        for (int p0 = 0; p0 < Up; p0 += 8) {
+#pragma unroll
+          for (int r = 0; r < 8; ++r) c_fma(G[r], sr[p0 + r], tw[(size_t)(p0 + r) * Qx]);
+        }
+        idft8(G);
+        float2* o = rows + (size_t)vi * Fx + b;
+#pragma unroll
+        for (int a = 0; a < 8; ++a) o[a * Qx] = G[a];
+      }
+  }
+  __syncthreads();
+  float2* out = BATCH ? outs[e.x] : out_one;
+  switch (Vp >> 3) {
+    case 1: fused_y<1, TILED>(it, rows, twy, f, c, ys, ysplit, out); break;
+    case 2: fused_y<2, TILED>(it, rows, twy, f, c, ys, ysplit, out); break;
+    case 3: if constexpr (NGM >= 3) fused_y<3, TILED>(it, rows, twy, f, c, ys, ysplit, out); break;
+    case 4: if constexpr (NGM >= 6) fused_y<4, TILED>(it, rows, twy, f, c, ys, ysplit, out); break;
+    case 5: if constexpr (NGM >= 6) fused_y<5, TILED>(it, rows, twy, f, c, ys, ysplit, out); break;
+    case 6: if constexpr (NGM >= 6) fused_y<6, TILED>(it, rows, twy, f, c, ys, ysplit, out); break;
+  }
+  if (one.trace) {
+    __syncthreads();
+    trace_end(one.trace, TRACE_YPASS);
+  }
+}
+
 // Fold + radix-8 inverse DFT along y of one tile from its rows in shared memory, and the field stores.
 // twy: the item's fold twiddles [Fy/8][Vp] (staged in shared memory, or the global table).
-template <bool BATCH, bool PAIR, bool TILED>
+template <bool BATCH, bool TILED>
 __device__ __forceinline__ void ypass_tile(const ItemDev& it, const float4* ys_col4, const float2* twy, int2 e, int c,
                                            int xb, float2* out_one, float2* const* outs) {
   const int f = e.y;
@@ -276,32 +542,6 @@ __device__ __forceinline__ void ypass_tile(const ItemDev& it, const float4* ys_c
     return;
   float2* dst = out + obase;
   const float4* col = ys_col4 + lane;
-  if constexpr (!PAIR) {
-    for (int b = w; b < Q; b += 8) {
-      const float4* tw = reinterpret_cast<const float4*>(twy + (size_t)b * Vp);  // twiddle pairs (Vp % 8 == 0)
-      float2 G0[8], G1[8];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) G0[r] = G1[r] = make_float2(0.f, 0.f);
-      for (int p0 = 0; p0 < Vp; p0 += 8) {
-#pragma unroll
-        for (int r = 0; r < 8; r += 2) {
-          const float4 tt = tw[(p0 + r) >> 1];
-          const float2 t0 = make_float2(tt.x, tt.y), t1 = make_float2(tt.z, tt.w);
-          const float4 d0 = col[(size_t)(p0 + r) * 32], d1 = col[(size_t)(p0 + r + 1) * 32];
-          c_fma(G0[r], make_float2(d0.x, d0.y), t0);
-          c_fma(G1[r], make_float2(d0.z, d0.w), t0);
-          c_fma(G0[r + 1], make_float2(d1.x, d1.y), t1);
-          c_fma(G1[r + 1], make_float2(d1.z, d1.w), t1);
-        }
-      }
-      idft8(G0);
-      idft8(G1);
-#pragma unroll
-      for (int a = 0; a < 8; ++a)
-        store_row4<TILED>(it, dst, b + a * Q, make_float4(G0[a].x, G0[a].y, G1[a].x, G1[a].y));
-    }
-    return;
-  }
   for (int b = w; b < Q; b += 16) {
     const bool two = b + 8 < Q;
     const float4* twA = reinterpret_cast<const float4*>(twy + (size_t)b * Vp);  // twiddle pairs
@@ -347,10 +587,8 @@ __device__ __forceinline__ void ypass_tile(const ItemDev& it, const float4* ys_c
 // a tile sit at their fold positions in shared memory ([Vp][64], padding rows zero);
 // two buffers: the rows of the CTA's next tile are copied in (cp.async) while the
 // current tile is folded and stored, so no CTA waits on its loads between tiles.
-// Lane l owns the column pair (2l, 2l+1). PAIR: warp w takes the residue pairs
-// (b, b + 8), b = w, w + 16, ..., so each shared-memory load feeds four complex FMAs
-// (long folds); otherwise one residue b = w, w + 8, ... at a time and twice the
-// resident warps (short folds, where latency dominates).
+// Lane l owns the column pair (2l, 2l+1); warp w takes the residue pairs (b, b + 8), b = w, w + 16, ...,
+// so each shared-memory load feeds four complex FMAs. For folds too long for registers (Vp > kYregMaxVp).
 template <bool BATCH, bool STW>
 __device__ __forceinline__ void ypass_prefetch(const ItemDev& one, const ItemDev* items, const int2* entries,
                                                int t, int n_tiles, int nxb, int rows_f4, float4* buf) {
@@ -380,8 +618,8 @@ __device__ __forceinline__ void ypass_prefetch(const ItemDev& one, const ItemDev
 }
 
 // STW: the fold twiddles travel with the rows into shared memory (when the largest table fits).
-template <bool BATCH, bool PAIR, bool TILED, bool STW>
-__global__ void __launch_bounds__(256, PAIR ? 2 : 4) ypass_kernel(const __grid_constant__ ItemDev one,
+template <bool BATCH, bool TILED, bool STW>
+__global__ void __launch_bounds__(256, 2) ypass_kernel(const __grid_constant__ ItemDev one,
                                                        const ItemDev* __restrict__ items,
                                                        const int2* __restrict__ entries, int n_tiles, int nxb,
                                                        int rows_f4, int buf_f4, float2* out_one,
@@ -403,7 +641,7 @@ __global__ void __launch_bounds__(256, PAIR ? 2 : 4) ypass_kernel(const __grid_c
     const ItemDev& it = BATCH ? items[e.x] : one;
     if (xb < it.Fx) {
       const float4* cur = ys_buf + (size_t)b * buf_f4;
-      ypass_tile<BATCH, PAIR, TILED>(it, cur, STW ? reinterpret_cast<const float2*>(cur + rows_f4) : it.twy, e, c,
+      ypass_tile<BATCH, TILED>(it, cur, STW ? reinterpret_cast<const float2*>(cur + rows_f4) : it.twy, e, c,
                                      xb, out_one, outs);
     }
     __syncthreads();          // buffer b is free for the prefetch of the next iteration
@@ -449,18 +687,18 @@ cudaError_t launch_xpass(const ItemDev& one, const ItemDev* items, const int2* d
 
 constexpr int kYpassTwiddleF4 = 1024;  // fold twiddles staged in shared memory up to 16 KB per table
 
-template <bool PAIR, bool TILED, bool STW>
-static cudaError_t launch_ypass_t(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
-                                  int max_Qx, int max_Vp, int tw_f4, float2* out_one, float2* const* d_outs,
-                                  cudaStream_t st) {
+template <bool TILED, bool STW>
+static cudaError_t launch_ypass_long(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
+                                     int max_Qx, int max_Vp, int tw_f4, float2* out_one, float2* const* d_outs,
+                                     cudaStream_t st) {
   const int nxb = (max_Qx * 8 + 63) / 64;
   const long long tiles = (long long)nxb * n_entries * 3;
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int rows_f4 = max_Vp * 32;
   const int buf_f4 = rows_f4 + (STW ? tw_f4 : 0);
   const size_t smem = 2 * (size_t)buf_f4 * sizeof(float4);
-  const void* fn = items ? reinterpret_cast<const void*>(ypass_kernel<true, PAIR, TILED, STW>)
-                         : reinterpret_cast<const void*>(ypass_kernel<false, PAIR, TILED, STW>);
+  const void* fn = items ? reinterpret_cast<const void*>(ypass_kernel<true, TILED, STW>)
+                         : reinterpret_cast<const void*>(ypass_kernel<false, TILED, STW>);
   cudaError_t e = allow_max_smem(fn);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
@@ -470,47 +708,111 @@ static cudaError_t launch_ypass_t(const ItemDev& one, const ItemDev* items, cons
   if (e != cudaSuccess) return e;
   const int grid = (int)std::min<long long>(tiles, (long long)std::max(1, per_sm) * sms);
   if (items)
-    return launch_pdl(ypass_kernel<true, PAIR, TILED, STW>, dim3(grid), dim3(256), smem, st, one, items, d_entries,
+    return launch_pdl(ypass_kernel<true, TILED, STW>, dim3(grid), dim3(256), smem, st, one, items, d_entries,
                       (int)tiles, nxb, rows_f4, buf_f4, (float2*)nullptr, d_outs);
-  return launch_pdl(ypass_kernel<false, PAIR, TILED, STW>, dim3(grid), dim3(256), smem, st, one,
-                    (const ItemDev*)nullptr, d_entries, (int)tiles, nxb, rows_f4, buf_f4, out_one,
-                    (float2* const*)nullptr);
+  return launch_pdl(ypass_kernel<false, TILED, STW>, dim3(grid), dim3(256), smem, st, one, (const ItemDev*)nullptr,
+                    d_entries, (int)tiles, nxb, rows_f4, buf_f4, out_one, (float2* const*)nullptr);
 }
 
-template <bool PAIR>
-static cudaError_t launch_ypass_p(bool tiled, const ItemDev& one, const ItemDev* items, const int2* d_entries,
-                                  int n_entries, int max_Qx, int max_Vp, int tw_f4, float2* out_one,
-                                  float2* const* d_outs, cudaStream_t st) {
-  const bool stw = tw_f4 <= kYpassTwiddleF4;
-#define SCW_YP(T, S) \
-  launch_ypass_t<PAIR, T, S>(one, items, d_entries, n_entries, max_Qx, max_Vp, tw_f4, out_one, d_outs, st)
-  if (tiled) return stw ? SCW_YP(true, true) : SCW_YP(true, false);
-  return stw ? SCW_YP(false, true) : SCW_YP(false, false);
-#undef SCW_YP
+template <bool BATCH, bool TILED, bool STW, int NGM>
+static cudaError_t launch_ypass_reg(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
+                                    int max_Qx, int tw_f4, float2* out_one, float2* const* d_outs, cudaStream_t st) {
+  const int nxb = (max_Qx * 8 + 63) / 64;
+  const long long tiles = (long long)nxb * n_entries * 3;
+  const size_t smem = STW ? (size_t)tw_f4 * sizeof(float4) : 0;
+  const void* fn = reinterpret_cast<const void*>(ypass_reg_kernel<BATCH, TILED, STW, NGM>);
+  int dev = 0, sms = 0, per_sm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kYregThreads, smem);
+  if (e != cudaSuccess) return e;
+  const long long warps = (long long)std::max(1, per_sm) * sms * (kYregThreads / 32);
+  // warps per tile: fewer read each x-pass row fewer times, more even out the last round
+  int rs = 4;
+  while (rs > 1 && tiles * (rs / 2) >= 8 * warps) rs /= 2;
+  const long long shares = tiles * rs;
+  if (shares > 0x7fffffffLL) return cudaErrorInvalidValue;
+  const int grid = (int)std::min<long long>((shares + kYregThreads / 32 - 1) / (kYregThreads / 32),
+                                            (long long)std::max(1, per_sm) * sms);
+  return launch_pdl(ypass_reg_kernel<BATCH, TILED, STW, NGM>, dim3(grid), dim3(kYregThreads), smem, st, one, items,
+                    d_entries, (int)shares, nxb, rs, out_one, d_outs);
 }
 
-// Pairs pay where the fold is long enough for the saved shared-memory loads to outweigh the halved
-// occupancy: measured on 21 x 21 orders (Vp = 24), one residue per warp is 3 us faster per
-// 256^3 step (and 0.08 ms per 128-item sweep), so pairs start at Vp = 32.
-bool ypass_pairs(int Vp) { return Vp >= 32; }
+bool ypass_long(int Vp) { return Vp > kYregMaxVp; }
 
-cudaError_t launch_ypass(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries, int n_pair,
+cudaError_t launch_ypass(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries, int n_long,
                          int max_Qx, int max_Vp, int max_twy, bool tiled, float2* out_one, float2* const* d_outs,
                          cudaStream_t st, int* launches) {
   const int tw_f4 = (max_twy + 1) / 2;
+  const bool stw = tw_f4 <= kYpassTwiddleF4;
   int n = 0;
   cudaError_t e = cudaSuccess;
-  if (n_pair > 0) {
-    e = launch_ypass_p<true>(tiled, one, items, d_entries, n_pair, max_Qx, max_Vp, tw_f4, out_one, d_outs, st);
+  if (n_long > 0) {
+#define SCW_YL(T, S) launch_ypass_long<T, S>(one, items, d_entries, n_long, max_Qx, max_Vp, tw_f4, out_one, d_outs, st)
+    e = tiled ? (stw ? SCW_YL(true, true) : SCW_YL(true, false)) : (stw ? SCW_YL(false, true) : SCW_YL(false, false));
+#undef SCW_YL
     ++n;
   }
-  if (e == cudaSuccess && n_entries > n_pair) {
-    e = launch_ypass_p<false>(tiled, one, items, d_entries + n_pair, n_entries - n_pair, max_Qx, max_Vp, tw_f4,
-                              out_one, d_outs, st);
+  if (e == cudaSuccess && n_entries > n_long) {
+    const int ngm = max_Vp <= 16 ? 2 : (max_Vp <= 24 ? 3 : 6);
+#define SCW_YR(B, T, S, G) \
+  launch_ypass_reg<B, T, S, G>(one, items, d_entries + n_long, n_entries - n_long, max_Qx, tw_f4, out_one, d_outs, st)
+#define SCW_YS(B, T, S) (ngm == 2 ? SCW_YR(B, T, S, 2) : ngm == 3 ? SCW_YR(B, T, S, 3) : SCW_YR(B, T, S, 6))
+    if (items)
+      e = tiled ? SCW_YS(true, true, false) : SCW_YS(true, false, false);
+    else if (stw)
+      e = tiled ? SCW_YS(false, true, true) : SCW_YS(false, false, true);
+    else
+      e = tiled ? SCW_YS(false, true, false) : SCW_YS(false, false, false);
+#undef SCW_YS
+#undef SCW_YR
     ++n;
   }
   if (launches) *launches = n;
   return e;
+}
+
+size_t fused_recompose_smem(int U, int V, int Fx, int Fy) {
+  const size_t b = fused_smem_bytes(U, V, Fx, Fy);
+  return (Fx > kFusedMaxFx || fold_np(V) > kYregMaxVp || b > 72 * 1024) ? 0 : b;  // three CTAs per SM
+}
+
+cudaError_t launch_recompose_fused(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
+                                   int max_Vp, size_t smem, bool tiled, float2* out_one, float2* const* d_outs,
+                                   cudaStream_t st) {
+  if (n_entries == 0) return cudaSuccess;
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const long long tiles = 3LL * n_entries;
+  const int ngm = max_Vp <= 16 ? 2 : (max_Vp <= 24 ? 3 : 6);
+  // The tiles of a last round that would leave most SMs with one CTA or two are split over the y residues
+  // (each part repeats the x-direction): `whole` tiles run one CTA each, the rest ysplit CTAs each. Splitting
+  // every tile in two costs 10 us of a 179 us step at 21 x 21 orders, 256^3; splitting none 10 us of 113 at
+  // 15 x 15 orders, 256^3 (768 tiles, four CTAs per SM), and 18 us of 54 at 21 x 21 orders and 24 planes.
+  const long long slots = (long long)sms * std::min<long long>(ngm == 2 ? 4 : 3, (227 * 1024) / ((long long)smem + 1024));
+  long long whole = tiles;
+  int ysplit = 1;
+  if (!items) {
+    const int Q = one.Fy >> 3, groups = std::max(1, kYregThreads / (one.Fx / (one.Vp <= 24 ? 2 : 1)));
+    const long long rest = tiles % slots;
+    const int most = tiles > slots ? 2 : 4;
+    while (rest > 0 && rest * ysplit < 2LL * sms && ysplit < most && Q >= 4 * groups * ysplit) ysplit *= 2;
+    if (ysplit > 1) whole = tiles - rest;
+  }
+  const long long grid = whole + (tiles - whole) * ysplit;
+  if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
+#define SCW_FU(B, T, G)                                                                                          \
+  [&]() -> cudaError_t {                                                                                         \
+    cudaError_t e = allow_max_smem(reinterpret_cast<const void*>(recompose_fused_kernel<B, T, G>));              \
+    if (e != cudaSuccess) return e;                                                                              \
+    return launch_pdl(recompose_fused_kernel<B, T, G>, dim3((unsigned)grid), dim3(kYregThreads), smem, st, one,   \
+                      items, d_entries, (int)whole, ysplit, out_one, d_outs);                                                                           \
+  }()
+#define SCW_FG(B, T) (ngm == 2 ? SCW_FU(B, T, 2) : ngm == 3 ? SCW_FU(B, T, 3) : SCW_FU(B, T, 6))
+  if (items) return tiled ? SCW_FG(true, true) : SCW_FG(true, false);
+  return tiled ? SCW_FG(false, true) : SCW_FG(false, false);
+#undef SCW_FG
+#undef SCW_FU
 }
 
 size_t recompose_smem_bytes(int V, int Up, int Vp) { return ((size_t)Vp * 64 + (size_t)V * Up) * sizeof(float2); }
