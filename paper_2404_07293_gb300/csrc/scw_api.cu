@@ -601,7 +601,7 @@ struct scw_plan_s {
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t gexec = nullptr;
   const void* graph_key = nullptr;
-  bool direct_done = false;
+  const void* seen_key = nullptr;  // output of the last directly launched call (run_synthesis)
   // timing
   bool timing = false;
   std::vector<cudaEvent_t> tev;
@@ -663,7 +663,7 @@ static void invalidate_graph(scw_plan_t P) {
   if (P->gexec) cudaGraphExecDestroy(P->gexec);
   P->gexec = nullptr;
   P->graph_key = nullptr;
-  P->direct_done = false;
+  P->seen_key = nullptr;
 }
 
 static scw_status upload_items(scw_plan_t P, cudaStream_t st) {
@@ -704,8 +704,11 @@ static scw_status enqueue_spectrum(scw_plan_t P, cudaStream_t st, bool marks, in
   const ItemDev& one = P->items[0]->item;
   const ItemDev* items = P->batched ? P->d_items : nullptr;
   mark(P, 0, st, marks);
+  // a single tensor-core plan's exterior planes are extra blocks of the phase kernel
+  const bool merged = P->tc && !P->batched && P->n_unit_entries > 0 && P->items[0]->n_exterior > 0;
   if (P->tc) {
-    e = launch_phases_tc(one, items, P->d_unit_entries, P->n_unit_entries, P->max_M, P->F_pad, P->bf16, st);
+    e = launch_phases_tc(one, items, P->d_unit_entries, P->n_unit_entries, P->max_M, P->F_pad, P->bf16,
+                         merged ? P->items[0] : nullptr, st);
     if (e != cudaSuccess) return cuda_error(e, "phase kernel launch");
     if (P->n_unit_entries) ++n;
   } else {
@@ -717,7 +720,7 @@ static scw_status enqueue_spectrum(scw_plan_t P, cudaStream_t st, bool marks, in
       }
   }
   for (auto* p : P->items)
-    if (p->n_exterior) {
+    if (p->n_exterior && !merged) {
       e = launch_exterior(*p, st);
       if (e != cudaSuccess) return cuda_error(e, "exterior kernel launch");
       ++n;
@@ -747,14 +750,10 @@ static scw_status enqueue_pipelined(scw_plan_t P, float2* out_one, cudaStream_t 
   cudaError_t e;
   Plan* p = P->items[0];
   const ItemDev& one = p->item;
-  e = launch_phases_tc(one, nullptr, P->d_unit_entries, P->n_unit_entries, P->max_M, P->F_pad, P->bf16, st);
+  e = launch_phases_tc(one, nullptr, P->d_unit_entries, P->n_unit_entries, P->max_M, P->F_pad, P->bf16,
+                       p->n_exterior ? p : nullptr, st);
   if (e != cudaSuccess) return cuda_error(e, "phase kernel launch");
   ++n;
-  if (p->n_exterior) {
-    e = launch_exterior(*p, st);
-    if (e != cudaSuccess) return cuda_error(e, "exterior kernel launch");
-    ++n;
-  }
   e = cudaEventRecord(P->ev_fork, st);  // st2 must not start before the previous step ended on st
   if (e != cudaSuccess) return cuda_error(e, "cudaEventRecord");
   e = cudaStreamWaitEvent(P->st2, P->ev_fork, 0);
@@ -817,9 +816,11 @@ static scw_status enqueue_synthesis(scw_plan_t P, float2* out_one, cudaStream_t 
   return SCW_OK;
 }
 
-// Timed launches go out directly (with events between kernels); otherwise the
-// first call for a given output launches directly and captures the same
-// sequence into a CUDA graph, later calls replay the graph.
+// Timed launches go out directly (with events between kernels). Otherwise the first call for a given
+// output launches directly, the second one captures the same sequence into a CUDA graph, and it and the
+// later calls replay the graph. Capturing and instantiating takes about 50 us of host time, longer than the
+// kernels of a mid-sized field: a program that brings a new solution (which drops the graph) or a new output
+// with every call never pays it.
 static scw_status run_synthesis(scw_plan_t P, float2* out_one, cudaStream_t st) {
   int n = 0;
   if (P->timing) {
@@ -828,32 +829,36 @@ static scw_status run_synthesis(scw_plan_t P, float2* out_one, cudaStream_t st) 
     return s;
   }
   const void* key = P->batched ? static_cast<const void*>(P->d_outs) : static_cast<const void*>(out_one);
-  if (P->gexec && P->graph_key == key) {
-    cudaError_t e = cudaGraphLaunch(P->gexec, st);
-    if (e != cudaSuccess) return cuda_error(e, "cudaGraphLaunch");
-    return SCW_OK;
+  cudaError_t e;
+  if (!(P->gexec && P->graph_key == key)) {
+    if (P->seen_key != key) {
+      scw_status s = enqueue_synthesis(P, out_one, st, false, n);
+      if (s != SCW_OK) return s;
+      P->kernels_per_synthesis = n;
+      P->seen_key = key;
+      return SCW_OK;
+    }
+    invalidate_graph(P);
+    cudaGraph_t g = nullptr;
+    e = cudaStreamBeginCapture(P->cap_stream, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return cuda_error(e, "cudaStreamBeginCapture");
+    scw_status s = enqueue_synthesis(P, out_one, P->cap_stream, false, n);
+    e = cudaStreamEndCapture(P->cap_stream, &g);
+    if (s != SCW_OK) {
+      if (g) cudaGraphDestroy(g);
+      return s;
+    }
+    if (e != cudaSuccess) return cuda_error(e, "cudaStreamEndCapture");
+    e = cudaGraphInstantiate(&P->gexec, g, 0);
+    cudaGraphDestroy(g);
+    if (e != cudaSuccess) {
+      P->gexec = nullptr;
+      return cuda_error(e, "cudaGraphInstantiate");
+    }
+    P->graph_key = key;
   }
-  scw_status s = enqueue_synthesis(P, out_one, st, false, n);
-  if (s != SCW_OK) return s;
-  P->kernels_per_synthesis = n;
-  invalidate_graph(P);
-  cudaGraph_t g = nullptr;
-  cudaError_t e = cudaStreamBeginCapture(P->cap_stream, cudaStreamCaptureModeThreadLocal);
-  if (e != cudaSuccess) return cuda_error(e, "cudaStreamBeginCapture");
-  s = enqueue_synthesis(P, out_one, P->cap_stream, false, n);
-  e = cudaStreamEndCapture(P->cap_stream, &g);
-  if (s != SCW_OK) {
-    if (g) cudaGraphDestroy(g);
-    return s;
-  }
-  if (e != cudaSuccess) return cuda_error(e, "cudaStreamEndCapture");
-  e = cudaGraphInstantiate(&P->gexec, g, 0);
-  cudaGraphDestroy(g);
-  if (e != cudaSuccess) {
-    P->gexec = nullptr;
-    return cuda_error(e, "cudaGraphInstantiate");
-  }
-  P->graph_key = key;
+  e = cudaGraphLaunch(P->gexec, st);
+  if (e != cudaSuccess) return cuda_error(e, "cudaGraphLaunch");
   return SCW_OK;
 }
 
@@ -1179,7 +1184,7 @@ static scw_status synthesize_host_pipelined(scw_plan_t P, const void* W, const v
       SCW_TRY_E(convert_w_layers(p, p->hio_W, P->hlayer[g], P->hlayer[g + 1], st), "W conversion launch");
     const int ub = P->hunit[g], nu = P->hunit[g + 1] - ub;
     if (nu > 0) {
-      SCW_TRY_E(launch_phases_tc(one, nullptr, P->d_unit_entries + ub, nu, P->max_M, P->F_pad, P->bf16, st),
+      SCW_TRY_E(launch_phases_tc(one, nullptr, P->d_unit_entries + ub, nu, P->max_M, P->F_pad, P->bf16, nullptr, st),
                 "phase kernel launch");
       SCW_TRY_E(launch_contract_tc(one, nullptr, P->hsched[g], P->NB, P->bf16, P->d_err, P->timeout_ns,
                                    P->inject_stall, st), "contraction kernel launch");

@@ -243,8 +243,9 @@ cudaError_t launch_convert_tiled(const float2* W, void* hi, void* lo, int L, int
 cudaError_t launch_transpose_layers(const float2* W, float2* Wt, int L, int rows, int cols, cudaStream_t st);
 
 // step (a): unit entries are (item, unit) pairs; items == nullptr means "the single item `one`"
+// (ext: a single plan whose exterior planes are evaluated by extra blocks of the same launch, or null)
 cudaError_t launch_phases_tc(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
-                             int max_M, int F_pad, bool bf16, cudaStream_t st);
+                             int max_M, int F_pad, bool bf16, const Plan* ext, cudaStream_t st);
 cudaError_t launch_phases_fp32(const Plan& p, cudaStream_t st);
 cudaError_t launch_exterior(const Plan& p, cudaStream_t st);
 

@@ -101,6 +101,65 @@ __device__ __forceinline__ size_t swz_offset(int n, int k, int rows) {
   return (size_t)kc * rows * 64 + (size_t)n * 64 + (size_t)(((g ^ (n & 7)) << 3) | (e & 7));
 }
 
+// Exterior planes (Eq. 9 with the reflected wave travelling towards -z):
+// S_part[0][f][c M + m]. Plane slot f carries illumination f mod I (p_* are [I][3][M]);
+// below the sample an optional pupil mask drops the orders outside the objective's NA.
+struct ExtArgs {
+  const int* planes;        // [n] plane slots outside [z0, zL]
+  int n;
+  double z0, zL, z_inc;
+  const double2 *sz_top, *sz_bot, *p_inc, *p_ref, *p_trn;
+  const float* pupil;
+};
+
+struct NoExt {};
+template <bool EXT> struct ExtOf { typedef NoExt T; };
+template <> struct ExtOf<true> { typedef ExtArgs T; };
+
+static ExtArgs ext_args(const Plan& p) {
+  return ExtArgs{p.d_ext_planes, p.n_exterior, p.z_bounds.front(), p.z_bounds.back(), p.z_inc, p.d_sz_top, p.d_sz_bot,
+                 p.p_inc, p.p_ref, p.p_trn, p.d_pupil};
+}
+
+__device__ __forceinline__ void exterior_order(const ExtArgs& a, const ItemDev& it, int f, int m) {
+  const double z = it.zplanes[f];
+  const int M = it.M;
+  float2* out = it.S_part + (size_t)f * 3 * M;
+  const size_t po = (size_t)(f % it.I) * 3 * M;
+  if (z < a.z0) {
+    const double2 st = a.sz_top[m];
+    const float2 gi = mode_factor(st, z - a.z_inc, it.inv_lam);
+    const float2 gr = mode_factor(st, -(z - a.z0), it.inv_lam);
+    for (int c = 0; c < 3; ++c) {
+      const double2 pi = a.p_inc[po + c * M + m], pr = a.p_ref[po + c * M + m];
+      const float2 x = cmulf(make_float2((float)pi.x, (float)pi.y), gi);
+      const float2 y = cmulf(make_float2((float)pr.x, (float)pr.y), gr);
+      if (in_bounds(it, BND_S_PART, (size_t)f * 3 * M + c * M + m)) out[c * M + m] = make_float2(x.x + y.x, x.y + y.y);
+    }
+  } else {
+    const double2 sb = a.sz_bot[m];
+    float2 gt = mode_factor(sb, z - a.zL, it.inv_lam);
+    if (a.pupil) gt = make_float2(gt.x * a.pupil[m], gt.y * a.pupil[m]);
+    for (int c = 0; c < 3; ++c) {
+      const double2 pt = a.p_trn[po + c * M + m];
+      if (in_bounds(it, BND_S_PART, (size_t)f * 3 * M + c * M + m))
+        out[c * M + m] = cmulf(make_float2((float)pt.x, (float)pt.y), gt);
+    }
+  }
+}
+
+// One block per (128 orders, exterior plane): batches and FP32 plans, and single plans whose planes are
+// all outside. A single tensor-core plan runs the same blocks behind those of phases_tc_kernel: its two
+// launches, one after the other, took 5.9 + 5.5 us at 12 layers of 15 x 13 orders and 6 planes outside.
+__global__ void __launch_bounds__(128) exterior_kernel(const __grid_constant__ ItemDev it,
+                                                       const __grid_constant__ ExtArgs a) {
+  trace_begin(it.trace, TRACE_EXTERIOR);
+  const int m = blockIdx.x * 128 + threadIdx.x;
+  if (m >= it.M) return;
+  exterior_order(a, it, a.planes[blockIdx.y], m);
+  trace_end(it.trace, TRACE_EXTERIOR);  // thread 0 always has an order (m = 128 blockIdx.x < M)
+}
+
 // B operand of the tensor-core contraction, per work unit nk chunks of NB rows
 // (NB = 2 F_pad) in the layout above: row f holds (Re c_j, -Im c_j) at columns
 // (2j, 2j+1), row F_pad + f holds (Im c_j, Re c_j); with A = W viewed as
@@ -114,12 +173,24 @@ __device__ __forceinline__ size_t swz_offset(int n, int k, int rows) {
 constexpr int kPhaseModes = 128;
 constexpr int kPhaseGroups = 1;
 
-template <typename T, bool BATCH>
+// EXT: blocks behind the units' evaluate the exterior planes of a single plan (a variant of its own: the
+// extra code and arguments cost 0.6 us of a 14 us step where there are none).
+template <typename T, bool BATCH, bool EXT>
 __global__ void __launch_bounds__(kPhaseModes * kPhaseGroups) phases_tc_kernel(const __grid_constant__ ItemDev one,
                                                                       const ItemDev* __restrict__ items,
-                                                                      const int2* __restrict__ entries, int F_pad) {
+                                                                      const int2* __restrict__ entries, int F_pad,
+                                                                      int n_entries,
+                                                                      const __grid_constant__ typename ExtOf<EXT>::T ext) {
   __shared__ PlaneOffsets off;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the contraction may start streaming W
+  if (EXT && (int)blockIdx.y >= n_entries) {  // exterior planes behind the units' blocks
+    const int m = blockIdx.x * kPhaseModes + threadIdx.x;
+    if (m >= one.M) return;
+    trace_begin(one.trace, TRACE_EXTERIOR);
+    if constexpr (EXT) exterior_order(ext, one, ext.planes[blockIdx.y - n_entries], m);
+    trace_end(one.trace, TRACE_EXTERIOR);
+    return;
+  }
   trace_begin(one.trace, TRACE_PHASES);
   const int2 e = entries[blockIdx.y];
   const ItemDev& it = BATCH ? items[e.x] : one;
@@ -222,49 +293,6 @@ __global__ void __launch_bounds__(128) phases_fp32_kernel(const LayerUnit* __res
   trace_end(trace, TRACE_PHASES);
 }
 
-// Exterior planes (Eq. 9 with the reflected wave travelling towards -z):
-// S_part[0][f][c M + m]. Plane slot f carries illumination f mod I (p_* are [I][3][M]);
-// below the sample an optional pupil mask drops the orders outside the objective's NA.
-__global__ void exterior_kernel(const int* __restrict__ ext_planes, const double* __restrict__ zplanes,
-                                double z0, double zL, double z_inc, const double2* __restrict__ sz_top,
-                                const double2* __restrict__ sz_bot, const double2* __restrict__ p_inc,
-                                const double2* __restrict__ p_ref, const double2* __restrict__ p_trn,
-                                int M, double inv_lam, float2* __restrict__ S, int I,
-                                const float* __restrict__ pupil, unsigned long long* trace,
-                                const __grid_constant__ ItemDev chk) {
-  trace_begin(trace, TRACE_EXTERIOR);
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= M) return;
-  const int f = ext_planes[blockIdx.y];
-  const double z = zplanes[f];
-  float2* out = S + (size_t)f * 3 * M;
-  const size_t po = (size_t)(f % I) * 3 * M;
-  p_inc += po;
-  p_ref += po;
-  p_trn += po;
-  if (z < z0) {
-    const double2 st = sz_top[m];
-    const float2 gi = mode_factor(st, z - z_inc, inv_lam);
-    const float2 gr = mode_factor(st, -(z - z0), inv_lam);
-    for (int c = 0; c < 3; ++c) {
-      const double2 a = p_inc[c * M + m], b = p_ref[c * M + m];
-      const float2 x = cmulf(make_float2((float)a.x, (float)a.y), gi);
-      const float2 y = cmulf(make_float2((float)b.x, (float)b.y), gr);
-      if (in_bounds(chk, BND_S_PART, (size_t)f * 3 * M + c * M + m)) out[c * M + m] = make_float2(x.x + y.x, x.y + y.y);
-    }
-  } else {
-    const double2 sb = sz_bot[m];
-    float2 gt = mode_factor(sb, z - zL, inv_lam);
-    if (pupil) gt = make_float2(gt.x * pupil[m], gt.y * pupil[m]);
-    for (int c = 0; c < 3; ++c) {
-      const double2 a = p_trn[c * M + m];
-      if (in_bounds(chk, BND_S_PART, (size_t)f * 3 * M + c * M + m))
-        out[c * M + m] = cmulf(make_float2((float)a.x, (float)a.y), gt);
-    }
-  }
-  trace_end(trace, TRACE_EXTERIOR);  // thread 0 always has an order (m = 128 blockIdx.x < M)
-}
-
 // ---- one-off conversions of W (plan time) -----------------------------------
 // W [L][R = 3M][K8 = 8M] reals (the complex64 layout) -> tile-major, swizzled
 // 16-bit copies for the tensor-core contraction: for layer l, row tile t
@@ -355,20 +383,24 @@ cudaError_t launch_transpose_layers(const float2* W, float2* Wt, int L, int rows
 
 template <typename T>
 static cudaError_t launch_phases_tc_t(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
-                                      int max_M, int F_pad, cudaStream_t st) {
-  dim3 grid((4 * max_M + kPhaseModes - 1) / kPhaseModes, n_entries);
+                                      int max_M, int F_pad, const Plan* ext, cudaStream_t st) {
+  const int threads = kPhaseModes * kPhaseGroups;
+  dim3 grid((4 * max_M + kPhaseModes - 1) / kPhaseModes, n_entries + (ext ? ext->n_exterior : 0));
   if (items)
-    phases_tc_kernel<T, true><<<grid, kPhaseModes * kPhaseGroups, 0, st>>>(one, items, d_entries, F_pad);
+    phases_tc_kernel<T, true, false><<<grid, threads, 0, st>>>(one, items, d_entries, F_pad, n_entries, NoExt{});
+  else if (ext)
+    phases_tc_kernel<T, false, true><<<grid, threads, 0, st>>>(one, nullptr, d_entries, F_pad, n_entries,
+                                                               ext_args(*ext));
   else
-    phases_tc_kernel<T, false><<<grid, kPhaseModes * kPhaseGroups, 0, st>>>(one, nullptr, d_entries, F_pad);
+    phases_tc_kernel<T, false, false><<<grid, threads, 0, st>>>(one, nullptr, d_entries, F_pad, n_entries, NoExt{});
   return cudaGetLastError();
 }
 
 cudaError_t launch_phases_tc(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
-                             int max_M, int F_pad, bool bf16, cudaStream_t st) {
+                             int max_M, int F_pad, bool bf16, const Plan* ext, cudaStream_t st) {
   if (n_entries == 0) return cudaSuccess;
-  return bf16 ? launch_phases_tc_t<__nv_bfloat16>(one, items, d_entries, n_entries, max_M, F_pad, st)
-              : launch_phases_tc_t<__half>(one, items, d_entries, n_entries, max_M, F_pad, st);
+  return bf16 ? launch_phases_tc_t<__nv_bfloat16>(one, items, d_entries, n_entries, max_M, F_pad, ext, st)
+              : launch_phases_tc_t<__half>(one, items, d_entries, n_entries, max_M, F_pad, ext, st);
 }
 
 cudaError_t launch_phases_fp32(const Plan& p, cudaStream_t st) {
@@ -383,11 +415,7 @@ cudaError_t launch_phases_fp32(const Plan& p, cudaStream_t st) {
 
 cudaError_t launch_exterior(const Plan& p, cudaStream_t st) {
   if (p.n_exterior == 0) return cudaSuccess;
-  dim3 grid((p.M + 127) / 128, p.n_exterior);
-  const double z0 = p.z_bounds.front(), zL = p.z_bounds.back();
-  exterior_kernel<<<grid, 128, 0, st>>>(p.d_ext_planes, p.d_zplanes, z0, zL, p.z_inc, p.d_sz_top, p.d_sz_bot,
-                                        p.p_inc, p.p_ref, p.p_trn, p.M, 1.0 / p.lambda, p.S_part, p.I, p.d_pupil,
-                                        p.item.trace, p.item);
+  exterior_kernel<<<dim3((p.M + 127) / 128, p.n_exterior), 128, 0, st>>>(p.item, ext_args(p));
   return cudaGetLastError();
 }
 
