@@ -594,6 +594,7 @@ struct scw_plan_s {
   float2** d_outs = nullptr;
   float2** h_outs = nullptr;       // pinned
   int max_M = 0, max_Qx = 0, max_V = 0, max_Vp = 0;
+  PhaseShape phase;
   size_t xpass_smem = 0;
   size_t fused_smem = 0;  // shared memory of the one-kernel recomposition; 0: x-pass and y-pass (fuse_recompose)
   size_t rec_smem = 0;
@@ -705,9 +706,10 @@ static scw_status enqueue_spectrum(scw_plan_t P, cudaStream_t st, bool marks, in
   const ItemDev* items = P->batched ? P->d_items : nullptr;
   mark(P, 0, st, marks);
   // a single tensor-core plan's exterior planes are extra blocks of the phase kernel
-  const bool merged = P->tc && !P->batched && P->n_unit_entries > 0 && P->items[0]->n_exterior > 0;
+  const bool merged = P->tc && !P->batched && P->n_unit_entries > 0 && P->items[0]->n_exterior > 0 &&
+                      P->phase.max_I == 1;
   if (P->tc) {
-    e = launch_phases_tc(one, items, P->d_unit_entries, P->n_unit_entries, P->max_M, P->F_pad, P->bf16,
+    e = launch_phases_tc(one, items, P->d_unit_entries, P->n_unit_entries, P->phase, P->bf16,
                          merged ? P->items[0] : nullptr, st);
     if (e != cudaSuccess) return cuda_error(e, "phase kernel launch");
     if (P->n_unit_entries) ++n;
@@ -750,10 +752,15 @@ static scw_status enqueue_pipelined(scw_plan_t P, float2* out_one, cudaStream_t 
   cudaError_t e;
   Plan* p = P->items[0];
   const ItemDev& one = p->item;
-  e = launch_phases_tc(one, nullptr, P->d_unit_entries, P->n_unit_entries, P->max_M, P->F_pad, P->bf16,
-                       p->n_exterior ? p : nullptr, st);
+  e = launch_phases_tc(one, nullptr, P->d_unit_entries, P->n_unit_entries, P->phase, P->bf16,
+                       p->n_exterior && p->I == 1 ? p : nullptr, st);
   if (e != cudaSuccess) return cuda_error(e, "phase kernel launch");
   ++n;
+  if (p->n_exterior && p->I > 1) {
+    e = launch_exterior(*p, st);
+    if (e != cudaSuccess) return cuda_error(e, "exterior kernel launch");
+    ++n;
+  }
   e = cudaEventRecord(P->ev_fork, st);  // st2 must not start before the previous step ended on st
   if (e != cudaSuccess) return cuda_error(e, "cudaEventRecord");
   e = cudaStreamWaitEvent(P->st2, P->ev_fork, 0);
@@ -1031,6 +1038,9 @@ static scw_status finish_plan(scw_plan_t P, const std::vector<int>& user_ks, boo
   for (size_t i = 0; i < P->items.size(); ++i) {
     Plan* p = P->items[i];
     for (int u = 0; u < (int)p->units.size(); ++u) ue.push_back(make_int2((int)i, u));
+    for (const LayerUnit& u : p->units)
+      P->phase.max_planes = std::max(P->phase.max_planes, (u.f0 + u.nf - 1) / p->I - u.f0 / p->I + 1);
+    P->phase.max_I = std::max(P->phase.max_I, p->I);
     for (int f = 0; f < p->Fz; ++f) pe.push_back(make_int2((int)i, f));
     P->max_M = std::max(P->max_M, p->M);
     P->max_Qx = std::max(P->max_Qx, p->Fx / 8);
@@ -1047,6 +1057,8 @@ static scw_status finish_plan(scw_plan_t P, const std::vector<int>& user_ks, boo
   P->n_long_entries = 0;
   for (const int2& en : pe) P->n_long_entries += ypass_long(P->items[en.x]->item.Vp) ? 1 : 0;
   P->fused_smem = fuse_recompose(P, (int)pe.size());
+  P->phase.max_M = P->max_M;
+  P->phase.F_pad = P->F_pad;
   P->n_unit_entries = (int)ue.size();
   P->n_plane_entries = (int)pe.size();
   SCW_TRY(upload(&P->d_unit_entries, ue, tot));
@@ -1184,7 +1196,7 @@ static scw_status synthesize_host_pipelined(scw_plan_t P, const void* W, const v
       SCW_TRY_E(convert_w_layers(p, p->hio_W, P->hlayer[g], P->hlayer[g + 1], st), "W conversion launch");
     const int ub = P->hunit[g], nu = P->hunit[g + 1] - ub;
     if (nu > 0) {
-      SCW_TRY_E(launch_phases_tc(one, nullptr, P->d_unit_entries + ub, nu, P->max_M, P->F_pad, P->bf16, nullptr, st),
+      SCW_TRY_E(launch_phases_tc(one, nullptr, P->d_unit_entries + ub, nu, P->phase, P->bf16, nullptr, st),
                 "phase kernel launch");
       SCW_TRY_E(launch_contract_tc(one, nullptr, P->hsched[g], P->NB, P->bf16, P->d_err, P->timeout_ns,
                                    P->inject_stall, st), "contraction kernel launch");

@@ -243,9 +243,15 @@ cudaError_t launch_convert_tiled(const float2* W, void* hi, void* lo, int L, int
 cudaError_t launch_transpose_layers(const float2* W, float2* Wt, int L, int rows, int cols, cudaStream_t st);
 
 // step (a): unit entries are (item, unit) pairs; items == nullptr means "the single item `one`"
-// (ext: a single plan whose exterior planes are evaluated by extra blocks of the same launch, or null)
+// (ext: a single plan of one illumination whose exterior planes are evaluated by extra blocks of the
+// same launch, or null)
+struct PhaseShape {
+  int max_M = 0, F_pad = 8;  // largest order count of the items, plane slots per unit
+  int max_I = 1;             // most illuminations of an item
+  int max_planes = 1;        // most output planes with slots in one unit
+};
 cudaError_t launch_phases_tc(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
-                             int max_M, int F_pad, bool bf16, const Plan* ext, cudaStream_t st);
+                             const PhaseShape& sh, bool bf16, const Plan* ext, cudaStream_t st);
 cudaError_t launch_phases_fp32(const Plan& p, cudaStream_t st);
 cudaError_t launch_exterior(const Plan& p, cudaStream_t st);
 

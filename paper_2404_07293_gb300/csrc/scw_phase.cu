@@ -173,6 +173,29 @@ __global__ void __launch_bounds__(128) exterior_kernel(const __grid_constant__ I
 constexpr int kPhaseModes = 128;
 constexpr int kPhaseGroups = 1;
 
+// Rows f (Re c, -Im c) and F_pad + f (Im c, Re c) of mode j's columns (2j, 2j + 1), hi and lo.
+template <typename T>
+__device__ __forceinline__ void store_b_pair(const ItemDev& it, size_t base, T* Bhi, T* Blo, int f, int j, int F_pad,
+                                             float2 cv) {
+  const int NB = 2 * F_pad;
+  const float v0[2] = {cv.x, -cv.y};
+  const float v1[2] = {cv.y, cv.x};
+  Pair<T> h0, l0, h1, l1;
+  h0.a = to_lp<T>(v0[0]); h0.b = to_lp<T>(v0[1]);
+  l0.a = to_lp<T>(v0[0] - from_lp<T>(h0.a)); l0.b = to_lp<T>(v0[1] - from_lp<T>(h0.b));
+  h1.a = to_lp<T>(v1[0]); h1.b = to_lp<T>(v1[1]);
+  l1.a = to_lp<T>(v1[0] - from_lp<T>(h1.a)); l1.b = to_lp<T>(v1[1] - from_lp<T>(h1.b));
+  const size_t i0 = swz_offset(f, 2 * j, NB), i1 = swz_offset(F_pad + f, 2 * j, NB);
+  if (in_bounds(it, BND_B, base + i0 + 1)) {  // a pair: its second element is the last one written
+    *reinterpret_cast<Pair<T>*>(Bhi + i0) = h0;
+    *reinterpret_cast<Pair<T>*>(Blo + i0) = l0;
+  }
+  if (in_bounds(it, BND_B, base + i1 + 1)) {
+    *reinterpret_cast<Pair<T>*>(Bhi + i1) = h1;
+    *reinterpret_cast<Pair<T>*>(Blo + i1) = l1;
+  }
+}
+
 // EXT: blocks behind the units' evaluate the exterior planes of a single plan (a variant of its own: the
 // extra code and arguments cost 0.6 us of a 14 us step where there are none).
 template <typename T, bool BATCH, bool EXT>
@@ -202,10 +225,9 @@ __global__ void __launch_bounds__(kPhaseModes * kPhaseGroups) phases_tc_kernel(c
   // the mode's constants are requested before the block waits for the plane offsets
   double2 g = make_double2(0.0, 0.0), al = make_double2(0.0, 0.0);
   const size_t lj = (size_t)u.layer * M4 + j;
-  const double2* alpha_lj = it.alpha + lj;  // illumination 0
   if (j < M4) {
     if (in_bounds(it, BND_GAMMA, lj)) g = it.gamma[lj];
-    if (in_bounds(it, BND_ALPHA, lj)) al = alpha_lj[0];
+    if (in_bounds(it, BND_ALPHA, lj)) al = it.alpha[lj];
   }
   load_offsets(off, u, it.zplanes, it.zbounds);
   __syncthreads();
@@ -221,33 +243,73 @@ __global__ void __launch_bounds__(kPhaseModes * kPhaseGroups) phases_tc_kernel(c
       if (f < u.nf) {
         const float dh = fwd ? off.f_hi[f] : off.b_hi[f];
         const float dl = fwd ? off.f_lo[f] : off.b_lo[f];
-        float2 a = mc.alpha;
-        if (it.I > 1) {  // plane slot f I + i carries illumination i
-          const size_t ia = (size_t)((u.f0 + f) % it.I) * it.alpha_istride;
-          const double2 ai = in_bounds(it, BND_ALPHA, lj + ia) ? alpha_lj[ia] : make_double2(0.0, 0.0);
-          a = make_float2((float)ai.x, (float)ai.y);
-        }
-        cv = cmulf(a, mode_factor_df(mc.a_hi, mc.a_lo, mc.c, dh, dl));
+        cv = cmulf(mc.alpha, mode_factor_df(mc.a_hi, mc.a_lo, mc.c, dh, dl));
       }
-      const float v0[2] = {cv.x, -cv.y};
-      const float v1[2] = {cv.y, cv.x};
-      Pair<T> h0, l0, h1, l1;
-      h0.a = to_lp<T>(v0[0]); h0.b = to_lp<T>(v0[1]);
-      l0.a = to_lp<T>(v0[0] - from_lp<T>(h0.a)); l0.b = to_lp<T>(v0[1] - from_lp<T>(h0.b));
-      h1.a = to_lp<T>(v1[0]); h1.b = to_lp<T>(v1[1]);
-      l1.a = to_lp<T>(v1[0] - from_lp<T>(h1.a)); l1.b = to_lp<T>(v1[1] - from_lp<T>(h1.b));
-      const size_t i0 = swz_offset(f, 2 * j, NB), i1 = swz_offset(F_pad + f, 2 * j, NB);
-      if (in_bounds(it, BND_B, base + i0 + 1)) {  // a pair: its second element is the last one written
-        *reinterpret_cast<Pair<T>*>(Bhi + i0) = h0;
-        *reinterpret_cast<Pair<T>*>(Blo + i0) = l0;
-      }
-      if (in_bounds(it, BND_B, base + i1 + 1)) {
-        *reinterpret_cast<Pair<T>*>(Bhi + i1) = h1;
-        *reinterpret_cast<Pair<T>*>(Blo + i1) = l1;
-      }
+      store_b_pair<T>(it, base, Bhi, Blo, f, j, F_pad, cv);
     }
   }
   trace_end(one.trace, TRACE_PHASES);  // thread 0 (mode kPhaseModes blockIdx.x < 4M) stamps after its planes
+}
+
+// The same operand for plans with I > 1 illuminations. The I slots of a plane share z, so a thread forms
+// the factors exp(i k gamma dz) of its mode once per plane (its own column of shared memory) and then
+// multiplies them by the amplitude of each of its kIllumGroup illuminations, loaded and rounded once: one
+// sincos, one exp and two FP64 conversions per slot, as in the kernel above, took 88 us of a 560 us step
+// at 16 illuminations (21 x 21 orders, 32 layers of 8 planes); with this kernel the step takes 503. Blocks are (mode block, unit
+// entry, illumination group). Slots past the unit's planes keep the zeros of plan creation.
+constexpr int kIllumGroup = 4;
+
+template <typename T, bool BATCH>
+__global__ void __launch_bounds__(kPhaseModes) phases_illum_kernel(const __grid_constant__ ItemDev one,
+                                                                   const ItemDev* __restrict__ items,
+                                                                   const int2* __restrict__ entries, int F_pad) {
+  __shared__ PlaneOffsets off;
+  extern __shared__ float2 fct[];  // [planes of the unit][kPhaseModes]
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the contraction may start streaming W
+  trace_begin(one.trace, TRACE_PHASES);
+  const int2 e = entries[blockIdx.y];
+  const ItemDev& it = BATCH ? items[e.x] : one;
+  const LayerUnit u = it.units[e.y];
+  const int M4 = 4 * it.M, I = it.I;
+  const int j = blockIdx.x * kPhaseModes + threadIdx.x;
+  const int i0 = blockIdx.z * kIllumGroup;
+  const size_t lj = (size_t)u.layer * M4 + j;
+  double2 g = make_double2(0.0, 0.0), al[kIllumGroup];
+#pragma unroll
+  for (int k = 0; k < kIllumGroup; ++k) {
+    al[k] = make_double2(0.0, 0.0);
+    const size_t ia = (size_t)(i0 + k) * it.alpha_istride + lj;
+    if (j < M4 && i0 + k < I && in_bounds(it, BND_ALPHA, ia)) al[k] = it.alpha[ia];
+  }
+  if (j < M4 && in_bounds(it, BND_GAMMA, lj)) g = it.gamma[lj];
+  load_offsets(off, u, it.zplanes, it.zbounds);
+  __syncthreads();
+  if (j < M4 && i0 < I) {
+    const ModeConst mc = mode_const(g, al[0], it.inv_lam);
+    const bool fwd = j < 2 * it.M;
+    // planes fo0 .. fo1 have slots in this unit; slot f = fo I + i - f0
+    const int fo0 = u.f0 / I, fo1 = (u.f0 + u.nf - 1) / I;
+    for (int fo = fo0; fo <= fo1; ++fo) {
+      const int f = max(fo * I - u.f0, 0);  // the plane's first slot here
+      fct[(fo - fo0) * kPhaseModes + threadIdx.x] =
+          mode_factor_df(mc.a_hi, mc.a_lo, mc.c, fwd ? off.f_hi[f] : off.b_hi[f], fwd ? off.f_lo[f] : off.b_lo[f]);
+    }
+    const int NB = 2 * F_pad;
+    const size_t base = (size_t)e.y * it.nk * NB * 64;  // B is per work unit
+    T* Bhi = static_cast<T*>(it.Bhi) + base;
+    T* Blo = static_cast<T*>(it.Blo) + base;
+    for (int fo = fo0; fo <= fo1; ++fo) {
+      const float2 x = fct[(fo - fo0) * kPhaseModes + threadIdx.x];
+#pragma unroll
+      for (int k = 0; k < kIllumGroup; ++k) {
+        const int f = fo * I + i0 + k - u.f0;
+        if (i0 + k >= I || f < 0 || f >= u.nf) continue;  // uniform over the block
+        const float2 cv = cmulf(make_float2((float)al[k].x, (float)al[k].y), x);
+        store_b_pair<T>(it, base, Bhi, Blo, f, j, F_pad, cv);
+      }
+    }
+  }
+  trace_end(one.trace, TRACE_PHASES);
 }
 
 // FP32 path: C[unit][j][f] complex64, plane index fastest; one thread per mode.
@@ -383,24 +445,39 @@ cudaError_t launch_transpose_layers(const float2* W, float2* Wt, int L, int rows
 
 template <typename T>
 static cudaError_t launch_phases_tc_t(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
-                                      int max_M, int F_pad, const Plan* ext, cudaStream_t st) {
+                                      const PhaseShape& sh, const Plan* ext, cudaStream_t st) {
   const int threads = kPhaseModes * kPhaseGroups;
-  dim3 grid((4 * max_M + kPhaseModes - 1) / kPhaseModes, n_entries + (ext ? ext->n_exterior : 0));
+  const unsigned gx = (4 * sh.max_M + kPhaseModes - 1) / kPhaseModes;
+  if (sh.max_I > 1) {
+    const dim3 grid(gx, n_entries, (sh.max_I + kIllumGroup - 1) / kIllumGroup);
+    const size_t smem = (size_t)sh.max_planes * kPhaseModes * sizeof(float2);
+    const void* fn = items ? reinterpret_cast<const void*>(phases_illum_kernel<T, true>)
+                           : reinterpret_cast<const void*>(phases_illum_kernel<T, false>);
+    cudaError_t e = allow_max_smem(fn);
+    if (e != cudaSuccess) return e;
+    if (items)
+      phases_illum_kernel<T, true><<<grid, kPhaseModes, smem, st>>>(one, items, d_entries, sh.F_pad);
+    else
+      phases_illum_kernel<T, false><<<grid, kPhaseModes, smem, st>>>(one, nullptr, d_entries, sh.F_pad);
+    return cudaGetLastError();
+  }
+  const dim3 grid(gx, n_entries + (ext ? ext->n_exterior : 0));
   if (items)
-    phases_tc_kernel<T, true, false><<<grid, threads, 0, st>>>(one, items, d_entries, F_pad, n_entries, NoExt{});
+    phases_tc_kernel<T, true, false><<<grid, threads, 0, st>>>(one, items, d_entries, sh.F_pad, n_entries, NoExt{});
   else if (ext)
-    phases_tc_kernel<T, false, true><<<grid, threads, 0, st>>>(one, nullptr, d_entries, F_pad, n_entries,
+    phases_tc_kernel<T, false, true><<<grid, threads, 0, st>>>(one, nullptr, d_entries, sh.F_pad, n_entries,
                                                                ext_args(*ext));
   else
-    phases_tc_kernel<T, false, false><<<grid, threads, 0, st>>>(one, nullptr, d_entries, F_pad, n_entries, NoExt{});
+    phases_tc_kernel<T, false, false><<<grid, threads, 0, st>>>(one, nullptr, d_entries, sh.F_pad, n_entries, NoExt{});
   return cudaGetLastError();
 }
 
 cudaError_t launch_phases_tc(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
-                             int max_M, int F_pad, bool bf16, const Plan* ext, cudaStream_t st) {
+                             const PhaseShape& sh, bool bf16, const Plan* ext, cudaStream_t st) {
   if (n_entries == 0) return cudaSuccess;
-  return bf16 ? launch_phases_tc_t<__nv_bfloat16>(one, items, d_entries, n_entries, max_M, F_pad, ext, st)
-              : launch_phases_tc_t<__half>(one, items, d_entries, n_entries, max_M, F_pad, ext, st);
+  if (ext != nullptr && sh.max_I > 1) return cudaErrorInvalidValue;  // that kernel has no exterior blocks
+  return bf16 ? launch_phases_tc_t<__nv_bfloat16>(one, items, d_entries, n_entries, sh, ext, st)
+              : launch_phases_tc_t<__half>(one, items, d_entries, n_entries, sh, ext, st);
 }
 
 cudaError_t launch_phases_fp32(const Plan& p, cudaStream_t st) {
