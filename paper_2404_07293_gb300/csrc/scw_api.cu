@@ -554,18 +554,6 @@ static std::vector<int> splits_for_target(const std::vector<Plan*>& items, int t
   return ks;
 }
 
-// FP32 path: ~4 waves of work units and a shared-memory slice of C <= 96 KB per CTA.
-static int fp32_split(const Plan* p) {
-  const int K = 4 * p->M;
-  const int slots = device_sms() * 2 * 4;
-  const int per_split_units = (int)p->units.size() * ((3 * p->M + 255) / 256);
-  int ks = per_split_units ? (slots + per_split_units - 1) / per_split_units : 1;
-  ks = std::max(1, std::min(ks, std::max(1, K / 128)));
-  const int fch = p->F_pad >= 16 ? 16 : 8;
-  ks = std::max(ks, (int)(((size_t)K * fch * 8 + 96 * 1024 - 1) / (96 * 1024)));
-  return std::min(ks, K);
-}
-
 }  // namespace scw
 
 using namespace scw;
@@ -879,7 +867,7 @@ static scw_status choose_splits(scw_plan_t P, bool timed, const std::vector<int>
   if (!P->tc) {
     for (size_t i = 0; i < P->items.size(); ++i) {
       Plan* p = P->items[i];
-      p->k_split = user_ks[i] > 0 ? user_ks[i] : fp32_split(p);
+      p->k_split = user_ks[i] > 0 ? user_ks[i] : fp32_split((int)p->units.size(), p->M, p->F_pad, device_sms());
       scw_status s = finish_item(p);
       if (s != SCW_OK) return s;
     }

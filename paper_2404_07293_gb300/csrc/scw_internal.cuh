@@ -261,6 +261,7 @@ cudaError_t launch_exterior(const Plan& p, cudaStream_t st);
 cudaError_t launch_contract_tc(const ItemDev& one, const ItemDev* items, const TcSchedule& s, int NB, bool bf16,
                                int* err, uint64_t timeout_ns, int inject, cudaStream_t st);
 cudaError_t launch_contract_fp32(const Plan& p, cudaStream_t st);
+int fp32_split(int n_units, int M, int F_pad, int sms);
 int tc_ctas_per_sm(int NB, bool bf16);
 
 // step (c): plane entries are (item, plane) pairs; S_override / nsplit_override replace the

@@ -322,6 +322,7 @@ __global__ void __launch_bounds__(128) phases_fp32_kernel(const LayerUnit* __res
                                                           size_t alpha_istride, unsigned long long* trace,
                                                           const __grid_constant__ ItemDev chk) {
   __shared__ PlaneOffsets off;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the contraction may start streaming W
   trace_begin(trace, TRACE_PHASES);
   const LayerUnit u = units[blockIdx.y];
   load_offsets(off, u, zplanes, zb);
