@@ -293,6 +293,7 @@ static scw_status reduce_all(scw_fno_s* f, std::vector<RedSeg>& segs, int B, cud
 template <typename T>
 static scw_status forward_backward(scw_fno_s* f, const float2* n, const float2* target, int B, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(f->grad, 0, (size_t)f->n_params * sizeof(float), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(f->loss_d, 0, 4 * sizeof(float), st);
   if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync");
   FNO_TRY(forward<T>(f, n, B, true, st));
   const int BC = B * C, P = f->P, nblk = f->nblk;
@@ -307,8 +308,6 @@ static scw_status forward_backward(scw_fno_s* f, const float2* n, const float2* 
   FNO_TRY(launch_ok(f, launch_head<T>(f->part_tn, f->part_err, f->part_pool, at<T>(f->wcopy, f->off_e), f->part_head,
                                       f->h_d, f->rel2_d, B, P, st),
                     "error head"));
-  e = cudaMemsetAsync(f->loss_d, 0, 4 * sizeof(float), st);
-  if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync");
   reduce_into(segs, f->part_head, B, C + 1, C + 3, f->grad + f->off_e);
   reduce_into(segs, f->part_head + C + 1, B, 2, C + 3, f->loss_d + 1);
   const long long ld = (long long)f->Bmax * C;

@@ -106,6 +106,7 @@ __global__ void __launch_bounds__(kDftThreads, 1) dft_modes_kernel(const __grid_
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     const uint32_t leader = ptx::elect_one();
+    pdl_sync();  // every result is stored behind loads issued after this
     int st = 0, issued = 0;
     uint32_t ph = 0;
     for (int t = blockIdx.x; t < n_tasks && !ptx::warp_any(abort_s); t += gridDim.x) {
@@ -319,9 +320,8 @@ static cudaError_t launch_dft_t(const CUtensorMap& mA, const CUtensorMap& mB, co
   if (e != cudaSuccess) return e;
   const int m_tiles = (M + 127) / 128, n_tiles = (N + BN - 1) / BN;
   const int grid = std::max(1, std::min(m_tiles * n_tiles, sms));
-  dft_modes_kernel<BN, DW><<<grid, kDftThreads, Cfg::SMEM, st>>>(mA, mB, mV, ea, ew, K, m_tiles, n_tiles, err,
-                                                                 timeout_ns);
-  return cudaGetLastError();
+  return launch_pdl(dft_modes_kernel<BN, DW>, dim3(grid), dim3(kDftThreads), Cfg::SMEM, st, mA, mB, mV, ea, ew, K,
+                    m_tiles, n_tiles, err, timeout_ns);
 }
 
 cudaError_t launch_dft_tc(const CUtensorMap& mA, const CUtensorMap* mB, const CUtensorMap* mV, const EpiArgs& ea,

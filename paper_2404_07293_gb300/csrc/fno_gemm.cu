@@ -114,6 +114,7 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_tc_kernel(const __grid_c
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     const uint32_t leader = ptx::elect_one();
+    pdl_sync();  // every result is stored behind loads issued after this
     int st = 0, issued = 0;
     uint32_t ph = 0;
     for (int i = 0; i < total && !ptx::warp_any(abort_s); ++i) {
@@ -358,6 +359,7 @@ __global__ void __launch_bounds__(kLayerThreads, 1) gemm_layer_persistent(const 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     const uint32_t leader = ptx::elect_one();
+    pdl_sync();  // every result is stored behind loads issued after this
     int st = 0, issued = 0;
     uint32_t ph = 0;
     for (int t = blockIdx.x; t < n_tasks && !ptx::warp_any(abort_s); t += gridDim.x) {
@@ -590,8 +592,8 @@ static cudaError_t launch_tc_t(const CUtensorMap& mA, const CUtensorMap& mB, con
   const int kper = (nkb + splits - 1) / splits;
   const dim3 grid((N + BN - 1) / BN, (M + 127) / 128, splits);
   if (grid.y > 65535u) return cudaErrorInvalidValue;
-  gemm_tc_kernel<BN, EPI><<<grid, kGemmThreads, Cfg::SMEM, st>>>(mA, mB, mA2, mW, ea, K, kper, err, timeout_ns);
-  return cudaGetLastError();
+  return launch_pdl(gemm_tc_kernel<BN, EPI>, grid, dim3(kGemmThreads), Cfg::SMEM, st, mA, mB, mA2, mW, ea, K, kper,
+                    err, timeout_ns);
 }
 
 template <int EPI>
@@ -605,9 +607,8 @@ static cudaError_t launch_layer_persistent(const CUtensorMap& mA, const CUtensor
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int m_tiles = (M + 127) / 128, n_tiles = (N + 255) / 256;
   const int grid = std::max(1, std::min(m_tiles * n_tiles, sms));
-  gemm_layer_persistent<EPI><<<grid, kLayerThreads, kLayerSmem, st>>>(mA, mB, mA2, mW, ea, K, m_tiles, n_tiles, err,
-                                                                      timeout_ns);
-  return cudaGetLastError();
+  return launch_pdl(gemm_layer_persistent<EPI>, dim3(grid), dim3(kLayerThreads), kLayerSmem, st, mA, mB, mA2, mW, ea, K,
+                    m_tiles, n_tiles, err, timeout_ns);
 }
 
 template <int EPI>

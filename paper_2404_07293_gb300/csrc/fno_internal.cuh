@@ -17,6 +17,15 @@ namespace fno {
 
 constexpr int C = 32;    // channels (width)
 constexpr int OUT = 6;   // Re/Im of E_x, E_y, E_z
+// The surrogate's kernels are launched programmatically dependent on their predecessor: a kernel's CTAs start
+// (barriers, tensor memory, descriptors) while it still runs, and pdl_sync waits for its results before
+// the first access that could see or disturb them. Its own successor is released only after that wait,
+// so whatever runs before the wait may rely on everything but the direct predecessor.
+__device__ __forceinline__ void pdl_sync() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 constexpr int PIX_BLOCK = 256;  // pixels per block of the per-pixel kernels (N*N is a multiple)
 
 // GEMM epilogues. Rows / columns are those of the GEMM's D = A B^T.

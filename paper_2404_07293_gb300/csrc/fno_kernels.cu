@@ -68,6 +68,7 @@ template <typename T>
 __global__ void __launch_bounds__(256, 3) lift_kernel(const float2* __restrict__ n, const T* __restrict__ prm,
                                                    T* __restrict__ Vcf, T* __restrict__ Vcl, int B, int S,
                                                    int in_grid, int N) {
+  pdl_sync();
   __shared__ __align__(16) float Ps[C * 32];  // [c][32], zero-padded past 2S
   __shared__ float ps[C];
   const int cin = 2 * S;
@@ -437,6 +438,7 @@ __global__ void transpose_w_kernel(const T* __restrict__ wcopy, long long off_W0
 // part_tn[b][blk] = sum over the block's pixels of |T|^2
 __global__ void __launch_bounds__(256) target_norm_kernel(const float2* __restrict__ target, float* __restrict__ part,
                                                           int P) {
+  pdl_sync();
   __shared__ float red[8];
   const int b = blockIdx.y, p = blockIdx.x * PIX_BLOCK + threadIdx.x;
   float s = 0.f;
@@ -469,6 +471,7 @@ __global__ void __launch_bounds__(256, 2) project_train_kernel(const T* __restri
                                                                float* __restrict__ part_err,
                                                                float* __restrict__ part_pool,
                                                                float* __restrict__ part_proj, int B, int P) {
+  pdl_sync();
   __shared__ __align__(16) float Qs[OUT * C + OUT];
   // the block sums below are one product F' V' over the block's pixels: F' = (dF rows, a row of
   // ones, a zero row), V' = (V columns, a column of ones, zero columns)
@@ -603,6 +606,7 @@ __global__ void __launch_bounds__(256) head_kernel(const float* __restrict__ par
                                                    const float* __restrict__ part_pool, const T* __restrict__ prm_e,
                                                    float* __restrict__ part_head, float* __restrict__ h_out,
                                                    float* __restrict__ rel2_out, int B, int nblk, int P) {
+  pdl_sync();
   const int lane = threadIdx.x & 31, b = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (b >= B) return;
   float pool = 0.f, tn = 0.f, e2 = 0.f;
@@ -639,6 +643,7 @@ __global__ void __launch_bounds__(256) head_kernel(const float* __restrict__ par
 template <typename T>
 __global__ void __launch_bounds__(128) lift_bwd_kernel(const T* __restrict__ dV0cl, const float2* __restrict__ n,
                                                        float* __restrict__ part, int B, int S, int in_grid, int N) {
+  pdl_sync();
   __shared__ __align__(16) float dv_s[128][C + 4];  // rows 16-byte aligned
   __shared__ __align__(16) float a_s[128][C + 4];   // features, zero past 2S
   __shared__ __align__(16) float red_s[128][16];
@@ -769,6 +774,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) project_infer_kernel(const T* __restrict__ Vcl, const T* __restrict__ prm_q,
                                                             float2* __restrict__ field, float* __restrict__ part_pool,
                                                             int P) {
+  pdl_sync();
   __shared__ __align__(16) float Qs[OUT * C + OUT];
   __shared__ float pool_s[PIX_BLOCK][C + 1];
   __shared__ float pool_w[8][C];
@@ -815,6 +821,7 @@ __global__ void __launch_bounds__(128) head_infer_kernel(const float* __restrict
                                                          const T* __restrict__ prm_e, float q, float threshold,
                                                          float* __restrict__ h_out, float* __restrict__ est,
                                                          unsigned char* __restrict__ flag, int B, int nblk, int P) {
+  pdl_sync();
   const int lane = threadIdx.x & 31, b = blockIdx.x * 4 + (threadIdx.x >> 5);
   if (b >= B) return;
   const float* src = part_pool + (size_t)b * nblk * C + lane;
@@ -849,8 +856,7 @@ template <typename T>
 cudaError_t launch_lift(const float2* n, const T* params, T* Vcf, T* Vcl, int B, int S, int in_grid, int N,
                         cudaStream_t st) {
   const long long total = (long long)B * in_grid * in_grid;
-  lift_kernel<T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(n, params, Vcf, Vcl, B, S, in_grid, N);
-  return cudaGetLastError();
+  return launch_pdl(lift_kernel<T>, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, n, params, Vcf, Vcl, B, S, in_grid, N);
 }
 
 template <typename T, int NM>
@@ -896,33 +902,27 @@ cudaError_t launch_transpose_w(const T* wcopy, long long off_W0, long long layer
 }
 
 cudaError_t launch_target_norm(const float2* target, float* part, int B, int P, cudaStream_t st) {
-  target_norm_kernel<<<dim3(P / PIX_BLOCK, B), PIX_BLOCK, 0, st>>>(target, part, P);
-  return cudaGetLastError();
+  return launch_pdl(target_norm_kernel, dim3(dim3(P / PIX_BLOCK, B)), dim3(PIX_BLOCK), 0, st, target, part, P);
 }
 
 template <typename T>
 cudaError_t launch_project_train(const T* Vcl, const float2* target, const T* params_q, const float* part_tn, T* dZcf,
                                  T* dZcl, float* part_err, float* part_pool, float* part_proj, int B, int P,
                                  cudaStream_t st) {
-  project_train_kernel<T><<<dim3(P / PIX_BLOCK, B), PIX_BLOCK, 0, st>>>(Vcl, target, params_q, part_tn, dZcf, dZcl,
-                                                                       part_err, part_pool, part_proj, B, P);
-  return cudaGetLastError();
+  return launch_pdl(project_train_kernel<T>, dim3(dim3(P / PIX_BLOCK, B)), dim3(PIX_BLOCK), 0, st, Vcl, target, params_q, part_tn, dZcf, dZcl, part_err, part_pool, part_proj, B, P);
 }
 
 template <typename T>
 cudaError_t launch_head(const float* part_tn, const float* part_err, const float* part_pool, const T* params_e,
                         float* part_head, float* h_out, float* rel2_out, int B, int P, cudaStream_t st) {
-  head_kernel<T><<<(B + 7) / 8, 256, 0, st>>>(part_tn, part_err, part_pool, params_e, part_head, h_out, rel2_out, B,
-                                              P / PIX_BLOCK, P);
-  return cudaGetLastError();
+  return launch_pdl(head_kernel<T>, dim3((B + 7) / 8), dim3(256), 0, st, part_tn, part_err, part_pool, params_e, part_head, h_out, rel2_out, B, P / PIX_BLOCK, P);
 }
 
 template <typename T>
 cudaError_t launch_lift_bwd(const T* dV0cl, const float2* n, float* part, int B, int S, int in_grid, int N,
                             cudaStream_t st) {
   const long long total = (long long)B * in_grid * in_grid;
-  lift_bwd_kernel<T><<<(unsigned)((total + 127) / 128), 128, 0, st>>>(dV0cl, n, part, B, S, in_grid, N);
-  return cudaGetLastError();
+  return launch_pdl(lift_bwd_kernel<T>, dim3((unsigned)((total + 127) / 128)), dim3(128), 0, st, dV0cl, n, part, B, S, in_grid, N);
 }
 
 // Segmented form of reduce_rows_kernel: block b belongs to the last segment whose first item is <= b.
@@ -934,6 +934,7 @@ __device__ __forceinline__ int find_segment(const RedSeg* segs, int nseg, int b,
 }
 
 __global__ void __launch_bounds__(256) reduce_segments_kernel(const RedSeg* __restrict__ segs, int nseg, int second) {
+  pdl_sync();
   __shared__ float red[8][33];
   const int b = blockIdx.x;
   const int si = find_segment(segs, nseg, b, second != 0);
@@ -1011,11 +1012,9 @@ bool plan_reduce_segments(std::vector<RedSeg>& segs, float* scratch, size_t scra
 
 cudaError_t launch_reduce_segments(const RedSeg* d_segs, int nseg, int items1, int items2, cudaStream_t st) {
   if (nseg == 0 || items1 == 0) return cudaSuccess;
-  reduce_segments_kernel<<<items1, dim3(32, 8), 0, st>>>(d_segs, nseg, 0);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(reduce_segments_kernel, dim3(items1), dim3(32, 8), 0, st, d_segs, nseg, 0);
   if (e != cudaSuccess || items2 == 0) return e;
-  reduce_segments_kernel<<<items2, dim3(32, 8), 0, st>>>(d_segs, nseg, 1);
-  return cudaGetLastError();
+  return launch_pdl(reduce_segments_kernel, dim3(items2), dim3(32, 8), 0, st, d_segs, nseg, 1);
 }
 
 // out[j] += scale * sum_r part[r pitch + j]; rows above 256 go through `scratch`
@@ -1052,16 +1051,13 @@ cudaError_t launch_copy_params(const float* master, T* copy, long long n, cudaSt
 template <typename T>
 cudaError_t launch_project_infer(const T* Vcl, const T* params_q, float2* field, float* part_pool, int B, int P,
                                  cudaStream_t st) {
-  project_infer_kernel<T><<<dim3(P / PIX_BLOCK, B), PIX_BLOCK, 0, st>>>(Vcl, params_q, field, part_pool, P);
-  return cudaGetLastError();
+  return launch_pdl(project_infer_kernel<T>, dim3(dim3(P / PIX_BLOCK, B)), dim3(PIX_BLOCK), 0, st, Vcl, params_q, field, part_pool, P);
 }
 
 template <typename T>
 cudaError_t launch_head_infer(const float* part_pool, const T* params_e, float q, float threshold, float* h_out,
                               float* est, unsigned char* flag, int B, int P, cudaStream_t st) {
-  head_infer_kernel<T><<<(B + 3) / 4, 128, 0, st>>>(part_pool, params_e, q, threshold, h_out, est, flag, B,
-                                                        P / PIX_BLOCK, P);
-  return cudaGetLastError();
+  return launch_pdl(head_infer_kernel<T>, dim3((B + 3) / 4), dim3(128), 0, st, part_pool, params_e, q, threshold, h_out, est, flag, B, P / PIX_BLOCK, P);
 }
 
 #define SCW_FNO_INSTANTIATE(T)                                                                                       \

@@ -69,6 +69,7 @@ __global__ void __launch_bounds__(256, 2) mix_tc_kernel(const float2* __restrict
     ptx::tmem_alloc(ptx::smem_u32(&tmem_base_s), kMixModes * 64);
     ptx::tmem_relinquish();
   }
+  pdl_sync();  // the spectra come from the preceding kernels
 
   // Operand loads: a thread stages 8 chunks of A (4 complex values each, one 16-byte chunk of BF16)
   // and 4 chunks of B. Every load it needs (R's words, then the first K-split partial of its A
@@ -271,6 +272,7 @@ __global__ void __launch_bounds__(256, 2) mix_dr_tc_kernel(const float2* __restr
     ptx::tmem_alloc(ptx::smem_u32(&tmem_base_s), 64);
     ptx::tmem_relinquish();
   }
+  pdl_sync();  // the spectra come from the preceding kernels
   // one work item: (mode mm, channel c = lane, quad of samples sq): its 4 samples' values of channel c
   // become one 16-byte K chunk (4 x (re, im)) of the rows for c. A thread has 8 items; the loads of
   // kDrBatch items are issued before any is used (the staging is bound by memory round trips).
@@ -415,11 +417,11 @@ cudaError_t launch_mix_dr_tc(const float2* G, const float2* V, int splits, long 
                              float* part, int B, int m, int N, int* err, uint64_t timeout_ns, cudaStream_t st) {
   if ((m * m) % kDrModes) return cudaErrorInvalidValue;
   const void* fn = reinterpret_cast<const void*>(mix_dr_tc_kernel);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDrSmem);
+  cudaError_t e = allow_max_smem(fn);
   if (e != cudaSuccess) return e;
   const dim3 grid(m * m / kDrModes, (B + kDrSamples - 1) / kDrSamples);
-  mix_dr_tc_kernel<<<grid, 256, kDrSmem, st>>>(G, V, splits, split_stride, ld, part, B, m, N, err, timeout_ns);
-  return cudaGetLastError();
+  return launch_pdl(mix_dr_tc_kernel, grid, dim3(256), kDrSmem, st, G, V, splits, split_stride, ld, part, B, m, N, err,
+                    timeout_ns);
 }
 
 cudaError_t launch_mix_tc(bool conj, const float2* X, int splits, long long split_stride, long long ld,
@@ -428,16 +430,11 @@ cudaError_t launch_mix_tc(bool conj, const float2* X, int splits, long long spli
   if ((m * m) % kMixModes || Kp % 8 || (ld % 2) || (split_stride % 2)) return cudaErrorInvalidValue;
   const void* fn = conj ? reinterpret_cast<const void*>(mix_tc_kernel<true>)
                         : reinterpret_cast<const void*>(mix_tc_kernel<false>);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMixSmem);
+  cudaError_t e = allow_max_smem(fn);
   if (e != cudaSuccess) return e;
   const dim3 grid(m * m / kMixModes, (B + kMixRows - 1) / kMixRows);
-  if (conj)
-    mix_tc_kernel<true><<<grid, 256, kMixSmem, st>>>(X, splits, split_stride, ld, R, out, scale, B, Kp, err,
-                                                     timeout_ns);
-  else
-    mix_tc_kernel<false><<<grid, 256, kMixSmem, st>>>(X, splits, split_stride, ld, R, out, scale, B, Kp, err,
-                                                      timeout_ns);
-  return cudaGetLastError();
+  return launch_pdl(conj ? mix_tc_kernel<true> : mix_tc_kernel<false>, grid, dim3(256), kMixSmem, st, X, splits,
+                    split_stride, ld, R, out, scale, B, Kp, err, timeout_ns);
 }
 
 }  // namespace fno

@@ -71,6 +71,7 @@ __global__ void points_table_fp32_kernel(const double2* __restrict__ xy, int P, 
 __global__ void points_spectrum_tc_kernel(const float2* __restrict__ S_part, size_t split_stride,
                                           const int* __restrict__ nsplit, int rows3, int M, int Kp,
                                           __nv_bfloat16* __restrict__ B) {
+  fno::pdl_sync();
   const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (i >= (size_t)rows3 * M) return;
   const int j = (int)(i / M), m = (int)(i - (size_t)j * M);
@@ -255,8 +256,8 @@ cudaError_t points_prepare(const PointTables& t, const Plan& p, cudaStream_t st)
   const size_t n = (size_t)t.rows3 * p.M;
   const size_t stride = (size_t)p.Fz * 3 * p.M;
   if (t.tc)
-    points_spectrum_tc_kernel<<<blocks_for(n, 256), 256, 0, st>>>(p.S_part, stride, p.d_nsplit, t.rows3, p.M, t.Kp,
-                                                                  static_cast<__nv_bfloat16*>(t.B));
+    return launch_pdl(points_spectrum_tc_kernel, dim3(blocks_for(n, 256)), dim3(256), 0, st, (const float2*)p.S_part,
+                      stride, (const int*)p.d_nsplit, t.rows3, p.M, t.Kp, static_cast<__nv_bfloat16*>(t.B));
   else
     points_spectrum_fp32_kernel<<<blocks_for(n, 256), 256, 0, st>>>(p.S_part, stride, p.d_nsplit, t.rows3, p.M,
                                                                     static_cast<float2*>(t.B));
