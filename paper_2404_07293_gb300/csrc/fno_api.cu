@@ -52,7 +52,7 @@ struct scw_fno_s {
   size_t scratch_floats = 0;
   // the backward pass's partial-sum reductions, all run by two launches at its end (per batch size)
   RedSeg* d_segs = nullptr;
-  int segs_B = -1, nseg = 0, seg_items1 = 0, seg_items2 = 0;
+  int segs_B = -1, segs_lift = 0, nseg = 0, seg_items1 = 0, seg_items2 = 0;
   float* loss_d = nullptr, *h_d = nullptr, *rel2_d = nullptr;
   int* d_err = nullptr;
   uint64_t timeout_ns = 2000000000ull;
@@ -269,9 +269,10 @@ static void reduce_into(std::vector<RedSeg>& segs, const float* part, int rows, 
   segs.push_back(sg);
 }
 
-// Every queued reduction in two launches; the table is uploaded when the batch size changes.
-static scw_status reduce_all(scw_fno_s* f, std::vector<RedSeg>& segs, int B, cudaStream_t st) {
-  if (f->segs_B != B) {
+// Every queued reduction in two launches; the table is uploaded when the batch size or the lift
+// backward's form changes.
+static scw_status reduce_all(scw_fno_s* f, std::vector<RedSeg>& segs, int B, int lift_rows, cudaStream_t st) {
+  if (f->segs_B != B || f->segs_lift != lift_rows) {
     if (!plan_reduce_segments(segs, f->scratch, f->scratch_floats, f->seg_items1, f->seg_items2))
       return set_error(SCW_ERR_UNSUPPORTED, "reduction scratch too small");
     if (f->d_segs) cudaFree(f->d_segs);
@@ -283,6 +284,7 @@ static scw_status reduce_all(scw_fno_s* f, std::vector<RedSeg>& segs, int B, cud
     if (e != cudaSuccess) return cuda_error(e, "reduction table");
     f->nseg = (int)segs.size();
     f->segs_B = B;
+    f->segs_lift = lift_rows;
   }
   cudaError_t e = launch_reduce_segments(f->d_segs, f->nseg, f->seg_items1, f->seg_items2, st);
   if (f->seg_items2) ++f->counter;
@@ -313,6 +315,7 @@ static scw_status forward_backward(scw_fno_s* f, const float2* n, const float2* 
   const long long ld = (long long)f->Bmax * C;
   const long long vstride = ld * (f->Kc / 2);
   const long long mix_w = (long long)f->m * f->m * C * C * 2;
+  const bool lift_cf = f->bf16 && lift_bwd_channel_first(n, f->S, f->in_grid, f->N);
   int cur = 0;
   for (int l = f->L - 1; l >= 0; --l) {
     const int ks = dft_splits(f, B), Kd = 2 * f->n_ind;
@@ -379,8 +382,9 @@ static scw_status forward_backward(scw_fno_s* f, const float2* n, const float2* 
     eb.w = at<T>(f->wcopy, f->off_W[l]);
     eb.x_cl = f->dZcl[cur];
     eb.g_in = l > 0 ? f->Gcl[l - 1] : nullptr;
-    eb.out_cf = l > 0 ? f->dZcf[1 - cur] : nullptr;  // dV_0 is consumed channel-last only (lift backward)
-    eb.out_cl = (!f->bf16 || l == 0) ? f->dZcl[1 - cur] : nullptr;
+    // dV_0 is consumed by the lift backward only, in the layout it reads
+    eb.out_cf = l > 0 || lift_cf ? f->dZcf[1 - cur] : nullptr;
+    eb.out_cl = (!f->bf16 || (l == 0 && !lift_cf)) ? f->dZcl[1 - cur] : nullptr;
     e = f->bf16 ? launch_gemm_tc(EPI_LAYER_BWD, 256, f->map_E, f->map_GVh, f->map_dZx[cur], f->map_WT[l], eb, P, BC,
                                  f->Kp, 1, f->d_err, f->timeout_ns, st)
                 : launch_gemm_simt(EPI_LAYER_BWD, static_cast<const float*>(f->E), f->Kp,
@@ -388,12 +392,12 @@ static scw_status forward_backward(scw_fno_s* f, const float2* n, const float2* 
     FNO_TRY(launch_ok(f, e, "layer backward", CAT_LAYER, 2.0 * P * BC * (f->Kc + C)));
     cur = 1 - cur;
   }
-  FNO_TRY(launch_ok(f, launch_lift_bwd<T>(static_cast<const T*>(f->dZcl[cur]), n, f->part_lift, B, f->S, f->in_grid,
-                                          f->N, st),
+  FNO_TRY(launch_ok(f, launch_lift_bwd<T>(static_cast<const T*>(lift_cf ? f->dZcf[cur] : f->dZcl[cur]), lift_cf, n,
+                                          f->part_lift, B, f->S, f->in_grid, f->N, st),
                     "lift backward"));
-  const int lift_rows = (B * f->in_grid * f->in_grid + 127) / 128;
+  const int lift_rows = lift_bwd_rows(lift_cf, B, f->in_grid);
   reduce_into(segs, f->part_lift, lift_rows, C * 2 * f->S + C, C * 2 * f->S + C, f->grad + f->off_P);
-  return reduce_all(f, segs, B, st);
+  return reduce_all(f, segs, B, lift_rows, st);
 }
 
 template <typename T>

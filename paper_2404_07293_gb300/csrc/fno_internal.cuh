@@ -391,9 +391,12 @@ cudaError_t launch_project_train(const T* Vcl, const float2* target, const T* pa
 template <typename T>
 cudaError_t launch_head(const float* part_tn, const float* part_err, const float* part_pool, const T* params_e,
                         float* part_head, float* h_out, float* rel2_out, int B, int P, cudaStream_t st);
+// dV_0 channel-first where lift_bwd_channel_first (BF16 mode), else channel-last; lift_bwd_rows(...) partial rows
+bool lift_bwd_channel_first(const float2* n, int S, int in_grid, int N);
+int lift_bwd_rows(bool channel_first, int B, int in_grid);
 template <typename T>
-cudaError_t launch_lift_bwd(const T* dV0cl, const float2* n, float* part, int B, int S, int in_grid, int N,
-                            cudaStream_t st);
+cudaError_t launch_lift_bwd(const T* dV0, bool channel_first, const float2* n, float* part, int B, int S, int in_grid,
+                            int N, cudaStream_t st);
 cudaError_t launch_reduce_rows_ex(const float* part, int rows, int width, long long pitch, float scale, float* out,
                                   float* scratch, cudaStream_t st);
 
@@ -408,7 +411,7 @@ struct RedSeg {
   long long pitch;
   int rows, width, ry, chunk;
   int item1, item2;  // first item of this segment in pass 1 (gx ry blocks) and pass 2 (gx blocks, ry > 1)
-  int wide;          // rows <= 8: each block takes 256 columns and each thread sums its column's rows
+  int wide;          // rows <= 8: each thread sums the rows of four columns
 };
 // Fills ry, chunk, item1, item2 and the scratch slices (from `scratch`, of `scratch_floats`);
 // returns false if the scratch is too small.
