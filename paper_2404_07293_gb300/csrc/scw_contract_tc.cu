@@ -312,6 +312,285 @@ __global__ void __launch_bounds__(192) contract_tc_kernel(const __grid_constant_
   }
 }
 
+// ---- 128 plane slots per unit (NB = 256) ----------------------------------------------------------------
+// A K chunk of B takes 64 KB of shared memory here, against 32 KB of A, and as one stage with A only two
+// fit: a chunk's B could be requested no earlier than one chunk ahead and took 1.2 us where its MMAs take
+// 0.8. So A and B have rings of their own, and B's is cut into halves of 128 columns, multiplied one after
+// the other (N = 128): four half chunks of B and three chunks of A (from memory) are in flight, and a half is
+// requested again as soon as its own MMAs are done. The same products in the same order. 16 illuminations
+// at 21 x 21 orders, 32 layers of 8 planes: 174 -> 161 us, 91 % of the tensor cores' rate under the power
+// cap. (Two row tiles per task, so that a B chunk is used twice, leave no tensor memory for a second set of
+// accumulators: 191 us.)
+template <bool SPLIT>
+struct RingCfg {
+  static constexpr int NB = 256, HB = 128;
+  static constexpr uint32_t A_TILE = 128u * 64u * 2u;
+  static constexpr int NA = SPLIT ? 2 : 1;
+  static constexpr uint32_t A_STAGE = NA * A_TILE;
+  static constexpr uint32_t B_HALF = (uint32_t)HB * 64u * 2u;  // hi or lo of half a chunk
+  static constexpr uint32_t B_STAGE = 2 * B_HALF;
+  static constexpr int BS = 4;
+  static constexpr int AS = SPLIT ? 3 : 6;
+  static constexpr uint32_t SMEM = BS * B_STAGE + AS * A_STAGE + 1024u;
+  static constexpr uint32_t TMEM_COLS = 512u;  // two accumulators
+};
+constexpr int kRingThreads = 320;
+
+template <bool SPLIT, bool BATCH>
+__global__ void __launch_bounds__(kRingThreads) contract_ring_kernel(const __grid_constant__ ItemDev one,
+                                                                     const ItemDev* __restrict__ items,
+                                                                     const int4* __restrict__ tasks,
+                                                                     const int* __restrict__ cta_off, int* err,
+                                                                     uint64_t timeout_ns, int inject_stall) {
+  using Cfg = RingCfg<SPLIT>;
+  constexpr int AS = Cfg::AS, BS = Cfg::BS, NB = Cfg::NB, NACC = 2;
+  constexpr int FP = NB / 2;  // plane slots
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t afull[AS], aempty[AS], bfull[BS], bempty[BS], accf_bar[NACC], acce_bar[NACC], drain_bar;
+  __shared__ uint32_t tmem_base_s;
+  __shared__ volatile int abort_s;
+
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem_a = smem + BS * Cfg::B_STAGE;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int t_begin = cta_off[blockIdx.x], t_end = cta_off[blockIdx.x + 1];
+  const uint64_t deadline = ptx::globaltimer() + timeout_ns;
+  ptx::griddep_launch_dependents();
+  trace_begin(one.trace, TRACE_CONTRACT);
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < AS; ++i) {
+      ptx::mbar_init(ptx::smem_u32(&afull[i]), 1);
+      ptx::mbar_init(ptx::smem_u32(&aempty[i]), 1);
+    }
+    for (int i = 0; i < BS; ++i) {
+      ptx::mbar_init(ptx::smem_u32(&bfull[i]), 1);
+      ptx::mbar_init(ptx::smem_u32(&bempty[i]), 1);
+    }
+    for (int i = 0; i < NACC; ++i) {
+      ptx::mbar_init(ptx::smem_u32(&accf_bar[i]), 1);
+      ptx::mbar_init(ptx::smem_u32(&acce_bar[i]), 8);  // one arrival per epilogue warp
+    }
+    ptx::mbar_init(ptx::smem_u32(&drain_bar), 1);
+    abort_s = 0;
+    ptx::fence_mbar_init();
+  }
+  if (warp == 0) {
+    ptx::tmem_alloc(ptx::smem_u32(&tmem_base_s), Cfg::TMEM_COLS);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = tmem_base_s;
+
+  if (warp == 0) {
+    // ---------------- bulk-copy producer ----------------
+    const uint32_t leader = ptx::elect_one();
+    const uint64_t pol_a = ptx::policy_evict_first(), pol_b = ptx::policy_evict_last();
+    int as = 0, bs = 0, a_issued = 0, b_issued = 0;
+    uint32_t aph = 0, bph = 0;
+    bool stalled = false, dep_done = false;  // stalled: failure injection, the first A chunk is never sent
+    for (int t = t_begin; t < t_end && !ptx::warp_any(abort_s); ++t) {
+      const int4 tk = tasks[t];
+      const ItemDev& it = BATCH ? items[tk.x] : one;
+      const TaskGeom g = task_geom(tk, it);
+      const size_t a0 = ((size_t)g.layer * 3 * it.M + (size_t)g.tile * it.rows_tile) * it.nk * 64;
+      const size_t b0 = (size_t)g.unit * it.nk * NB * 64;
+      const uint32_t a_bytes = (uint32_t)g.rt * 128u;
+      const uint16_t* Ah = static_cast<const uint16_t*>(it.Ahi);
+      const uint16_t* Al = static_cast<const uint16_t*>(it.Alo);
+      const uint16_t* Bh = static_cast<const uint16_t*>(it.Bhi);
+      const uint16_t* Bl = static_cast<const uint16_t*>(it.Blo);
+      for (int i = 0; i < g.kcount; ++i) {
+        const int kc = g.kb + i;
+        bool ok = ptx::mbar_wait_warp(ptx::smem_u32(&aempty[as]), aph ^ 1u, deadline);
+        if (ok) {
+          if (inject_stall && blockIdx.x == 0 && a_issued == 0) {
+            stalled = true;
+          } else {
+            const uint32_t fb = ptx::smem_u32(&afull[as]);
+            const uint32_t sa = ptx::smem_u32(smem_a + (size_t)as * Cfg::A_STAGE);
+            const size_t ao = a0 + (size_t)kc * g.rt * 64;
+            ptx::mbar_arrive_expect_tx(fb, Cfg::NA * a_bytes, leader);
+            ptx::bulk_load(sa, Ah + ao, a_bytes, fb, pol_a, leader);
+            if (SPLIT) ptx::bulk_load(sa + Cfg::A_TILE, Al + ao, a_bytes, fb, pol_a, leader);
+          }
+          ++a_issued;
+          if (++as == AS) {
+            as = 0;
+            aph ^= 1u;
+          }
+        }
+        // W does not depend on the phase kernel that precedes this grid (programmatic launch), B does
+        if (!dep_done) ptx::griddep_wait();
+        dep_done = true;
+        for (int h = 0; ok && h < 2; ++h) {
+          ok = ptx::mbar_wait_warp(ptx::smem_u32(&bempty[bs]), bph ^ 1u, deadline);
+          if (!ok) break;
+          const uint32_t fb = ptx::smem_u32(&bfull[bs]);
+          const uint32_t sb = ptx::smem_u32(smem + (size_t)bs * Cfg::B_STAGE);
+          const size_t bo = b0 + ((size_t)kc * NB + h * Cfg::HB) * 64;
+          ptx::mbar_arrive_expect_tx(fb, Cfg::B_STAGE, leader);
+          ptx::bulk_load(sb, Bh + bo, Cfg::B_HALF, fb, pol_b, leader);
+          ptx::bulk_load(sb + Cfg::B_HALF, Bl + bo, Cfg::B_HALF, fb, pol_b, leader);
+          ++b_issued;
+          if (++bs == BS) {
+            bs = 0;
+            bph ^= 1u;
+          }
+        }
+        if (!ok) {
+          if (leader) atomicOr(err, DEV_ERR_TIMEOUT_EMPTY);
+          abort_s = 1;
+          break;
+        }
+      }
+    }
+    if (!dep_done) ptx::griddep_wait();
+    if (ptx::warp_any(abort_s)) {
+      // let the last issued copies land before the CTA's shared memory goes away
+      const uint64_t d2 = ptx::drain_deadline(timeout_ns);
+      bool ok = true;
+      for (int back = 1; ok && back <= AS && back <= a_issued; ++back) {
+        const int i = a_issued - back;
+        if (stalled && i == 0) continue;  // nothing was sent to that stage
+        ok = ptx::mbar_wait_warp(ptx::smem_u32(&afull[i % AS]), (uint32_t)(i / AS) & 1u, d2);
+      }
+      for (int back = 1; ok && back <= BS && back <= b_issued; ++back) {
+        const int i = b_issued - back;
+        ok = ptx::mbar_wait_warp(ptx::smem_u32(&bfull[i % BS]), (uint32_t)(i / BS) & 1u, d2);
+      }
+      if (!ok && leader) atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
+    }
+  } else if (warp == 1) {
+    // ---------------- tcgen05.mma issuer ----------------
+    const uint32_t leader = ptx::elect_one();
+    constexpr uint32_t idesc = ptx::idesc_f16(SPLIT, 128, Cfg::HB);
+    int as = 0, bs = 0, lt = 0;
+    uint32_t aph = 0, bph = 0;
+    for (int t = t_begin; t < t_end && !ptx::warp_any(abort_s); ++t, ++lt) {
+      const int4 tk = tasks[t];
+      const ItemDev& it = BATCH ? items[tk.x] : one;
+      const TaskGeom g = task_geom(tk, it);
+      const int acc = lt % NACC;
+      if (!ptx::mbar_wait_warp(ptx::smem_u32(&acce_bar[acc]), ((uint32_t)(lt / NACC) & 1u) ^ 1u, deadline)) {
+        if (leader) atomicOr(err, DEV_ERR_TIMEOUT_ACCUM);
+        abort_s = 1;
+        break;
+      }
+      ptx::tc_fence_after();
+      bool ok = true;
+      for (int i = 0; i < g.kcount && ok; ++i) {
+        ok = ptx::mbar_wait_warp(ptx::smem_u32(&afull[as]), aph, deadline);
+        const uint32_t a_hi = ptx::smem_u32(smem_a + (size_t)as * Cfg::A_STAGE);
+        const uint64_t dah = ptx::sw128_desc(a_hi), dal = ptx::sw128_desc(a_hi + Cfg::A_TILE);
+        for (int h = 0; ok && h < 2; ++h) {
+          ok = ptx::mbar_wait_warp(ptx::smem_u32(&bfull[bs]), bph, deadline);
+          if (!ok) break;
+          ptx::tc_fence_after();
+          const uint32_t d_tmem = tmem + (uint32_t)(acc * NB + h * Cfg::HB);
+          const uint32_t b_hi = ptx::smem_u32(smem + (size_t)bs * Cfg::B_STAGE);
+          const uint64_t dbh = ptx::sw128_desc(b_hi), dbl = ptx::sw128_desc(b_hi + Cfg::B_HALF);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) {
+            const uint64_t o = (uint64_t)(2 * kk);
+            ptx::mma_f16(d_tmem, dah + o, dbh + o, idesc, (i > 0 || kk > 0) ? 1u : 0u, leader);
+            ptx::mma_f16(d_tmem, dah + o, dbl + o, idesc, 1u, leader);
+            if (SPLIT) ptx::mma_f16(d_tmem, dal + o, dbh + o, idesc, 1u, leader);
+          }
+          ptx::mma_commit(ptx::smem_u32(&bempty[bs]), leader);
+          if (++bs == BS) {
+            bs = 0;
+            bph ^= 1u;
+          }
+        }
+        if (!ok) break;
+        ptx::mma_commit(ptx::smem_u32(&aempty[as]), leader);
+        if (++as == AS) {
+          as = 0;
+          aph ^= 1u;
+        }
+      }
+      if (!ok) {
+        if (leader) atomicOr(err, DEV_ERR_TIMEOUT_FULL);
+        abort_s = 1;
+        break;
+      }
+      ptx::mma_commit(ptx::smem_u32(&accf_bar[acc]), leader);
+    }
+    if (ptx::warp_any(abort_s)) {
+      // issued MMAs must finish before the tensor memory is released
+      ptx::mma_commit(ptx::smem_u32(&drain_bar), leader);
+      if (!ptx::mbar_wait_warp(ptx::smem_u32(&drain_bar), 0u, ptx::drain_deadline(timeout_ns)))
+        if (leader) atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
+    }
+  } else {
+    // ---------------- epilogue: two warps per 32-lane quadrant, one per half of the planes ----------------
+    const int grp = warp & 3, h = (warp - 2) >> 2;  // TMEM lanes 32 grp .. 32 grp + 31
+    const uint64_t pol_s = ptx::policy_evict_last();
+    int lt = 0;
+    for (int t = t_begin; t < t_end; ++t, ++lt) {
+      const int4 tk = tasks[t];
+      const ItemDev& it = BATCH ? items[tk.x] : one;
+      const TaskGeom g = task_geom(tk, it);
+      const int acc = lt % NACC;
+      bool ok = true;
+      for (;;) {
+        if (ptx::mbar_try_wait(ptx::smem_u32(&accf_bar[acc]), (uint32_t)(lt / NACC) & 1u)) break;
+        if (abort_s || ptx::globaltimer() > deadline) {
+          ok = false;
+          break;
+        }
+      }
+      if (!__all_sync(0xffffffffu, ok)) {
+        if (lane == 0 && !abort_s) atomicOr(err, DEV_ERR_TIMEOUT_ACCUM);
+        abort_s = 1;
+        break;
+      }
+      ptx::tc_fence_after();
+      const int rows = 3 * it.M;
+      const int rl = grp * 32 + lane;  // row within the tile
+      const int row = g.tile * it.rows_tile + rl;
+      const size_t d0 = ((size_t)g.split * it.Fz + g.f0) * rows + row;
+      float2* dst = it.S_part + d0;
+      const uint32_t lane_addr = tmem + (uint32_t)(acc * NB) + ((uint32_t)(grp * 32) << 16);
+#pragma unroll 1
+      for (int f0 = h * (FP / 2); f0 < (h + 1) * (FP / 2) && f0 < g.nf; f0 += 8) {
+        uint32_t re[8], im[8];
+        if (g.kcount > 0) {
+          ptx::tmem_ld_x8(lane_addr + (uint32_t)f0, re);
+          ptx::tmem_ld_x8(lane_addr + (uint32_t)(FP + f0), im);
+          ptx::tmem_wait_ld();
+        } else {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) re[q] = im[q] = 0u;
+        }
+        if (rl < g.rt) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            if (f0 + q < g.nf && in_bounds(it, BND_S_PART, d0 + (size_t)(f0 + q) * rows))
+              ptx::st_global_hint(dst + (size_t)(f0 + q) * rows,
+                                  make_float2(__uint_as_float(re[q]), __uint_as_float(im[q])), pol_s);
+        }
+      }
+      ptx::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&acce_bar[acc]));
+    }
+  }
+
+  // ---------------- teardown ----------------
+  __syncwarp();
+  ptx::tc_fence_before();
+  __syncthreads();
+  trace_end(one.trace, TRACE_CONTRACT);
+  if (warp == 0) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem, Cfg::TMEM_COLS);
+  }
+}
+
 // ---------------------------------------------------------------- host side ---
 template <int NB, bool SPLIT>
 static cudaError_t launch_tc_t(const ItemDev& one, const ItemDev* items, const TcSchedule& s, int* err,
@@ -333,6 +612,16 @@ static cudaError_t launch_tc_t(const ItemDev& one, const ItemDev* items, const T
 }
 
 template <bool SPLIT>
+static cudaError_t launch_ring_t(const ItemDev& one, const ItemDev* items, const TcSchedule& s, int* err,
+                                 uint64_t timeout_ns, int inject, cudaStream_t st) {
+  auto fn = items ? contract_ring_kernel<SPLIT, true> : contract_ring_kernel<SPLIT, false>;
+  cudaError_t e = allow_max_smem(reinterpret_cast<const void*>(fn));
+  if (e != cudaSuccess) return e;
+  return launch_pdl(fn, dim3(s.grid), dim3(kRingThreads), RingCfg<SPLIT>::SMEM, st, one, items,
+                    (const int4*)s.d_tasks, (const int*)s.d_cta_off, err, timeout_ns, inject);
+}
+
+template <bool SPLIT>
 static cudaError_t launch_tc_nb(int NB, const ItemDev& one, const ItemDev* items, const TcSchedule& s, int* err,
                                 uint64_t timeout_ns, int inject, cudaStream_t st) {
   switch (NB) {
@@ -341,7 +630,7 @@ static cudaError_t launch_tc_nb(int NB, const ItemDev& one, const ItemDev* items
     case 48: return launch_tc_t<48, SPLIT>(one, items, s, err, timeout_ns, inject, st);
     case 64: return launch_tc_t<64, SPLIT>(one, items, s, err, timeout_ns, inject, st);
     case 128: return launch_tc_t<128, SPLIT>(one, items, s, err, timeout_ns, inject, st);
-    case 256: return launch_tc_t<256, SPLIT>(one, items, s, err, timeout_ns, inject, st);
+    case 256: return launch_ring_t<SPLIT>(one, items, s, err, timeout_ns, inject, st);
     default: return cudaErrorInvalidValue;
   }
 }
