@@ -164,14 +164,14 @@ __global__ void __launch_bounds__(128) exterior_kernel(const __grid_constant__ I
 // (NB = 2 F_pad) in the layout above: row f holds (Re c_j, -Im c_j) at columns
 // (2j, 2j+1), row F_pad + f holds (Im c_j, Re c_j); with A = W viewed as
 // interleaved reals this gives [Re S | Im S] (the complex product as one real
-// GEMM). hi = round(x), lo = round(x - hi). A block is kPhaseModes consecutive modes x
-// kPhaseGroups plane groups: thread t takes mode kPhaseModes blockIdx.x + t mod kPhaseModes and
-// the planes f = g, g + kPhaseGroups, ... (g = t / kPhaseModes) of its unit; every warp store
-// covers whole 128-byte rows. Blocks are (mode block, (item, unit) entry). One group (a thread
-// loops over all planes of its mode, whose constants it loads and reduces once) measured faster
-// than four (5.2 against 8.3 us per step at 21x21 orders, 32 layers of 8 planes).
+// GEMM). hi = round(x), lo = round(x - hi). Blocks are (kPhaseModes consecutive modes, (item, unit) entry,
+// kPhasePlanes plane slots), one thread per mode; every warp store covers whole 128-byte rows. A thread loads
+// and reduces its mode's constants once and loops over its planes: four threads of two planes each measured
+// slower for a unit of 8 planes (8.3 against 5.2 us per step at 21x21 orders, 32 layers), but the loop over
+// 64 or 128 slots is a chain of 10 to 18 us that the contraction waits for. In pieces of 16 slots, a whole
+// step at 23x7 orders, 2 layers of 100 planes: 39.5 -> 25.3 us.
+constexpr int kPhasePlanes = 16;
 constexpr int kPhaseModes = 128;
-constexpr int kPhaseGroups = 1;
 
 // Rows f (Re c, -Im c) and F_pad + f (Im c, Re c) of mode j's columns (2j, 2j + 1), hi and lo.
 template <typename T>
@@ -199,7 +199,7 @@ __device__ __forceinline__ void store_b_pair(const ItemDev& it, size_t base, T* 
 // EXT: blocks behind the units' evaluate the exterior planes of a single plan (a variant of its own: the
 // extra code and arguments cost 0.6 us of a 14 us step where there are none).
 template <typename T, bool BATCH, bool EXT>
-__global__ void __launch_bounds__(kPhaseModes * kPhaseGroups) phases_tc_kernel(const __grid_constant__ ItemDev one,
+__global__ void __launch_bounds__(kPhaseModes) phases_tc_kernel(const __grid_constant__ ItemDev one,
                                                                       const ItemDev* __restrict__ items,
                                                                       const int2* __restrict__ entries, int F_pad,
                                                                       int n_entries,
@@ -207,6 +207,7 @@ __global__ void __launch_bounds__(kPhaseModes * kPhaseGroups) phases_tc_kernel(c
   __shared__ PlaneOffsets off;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the contraction may start streaming W
   if (EXT && (int)blockIdx.y >= n_entries) {  // exterior planes behind the units' blocks
+    if (blockIdx.z > 0) return;
     const int m = blockIdx.x * kPhaseModes + threadIdx.x;
     if (m >= one.M) return;
     trace_begin(one.trace, TRACE_EXTERIOR);
@@ -219,8 +220,8 @@ __global__ void __launch_bounds__(kPhaseModes * kPhaseGroups) phases_tc_kernel(c
   const ItemDev& it = BATCH ? items[e.x] : one;
   const LayerUnit u = it.units[e.y];
   const int M = it.M;
-  const int j = blockIdx.x * kPhaseModes + (threadIdx.x % kPhaseModes);
-  const int fg = threadIdx.x / kPhaseModes;
+  const int j = blockIdx.x * kPhaseModes + threadIdx.x;
+  const int f_begin = blockIdx.z * kPhasePlanes, f_end = min(F_pad, f_begin + kPhasePlanes);
   const int M4 = 4 * M;
   // the mode's constants are requested before the block waits for the plane offsets
   double2 g = make_double2(0.0, 0.0), al = make_double2(0.0, 0.0);
@@ -238,7 +239,7 @@ __global__ void __launch_bounds__(kPhaseModes * kPhaseGroups) phases_tc_kernel(c
     const size_t base = (size_t)e.y * it.nk * NB * 64;  // B is per work unit
     T* Bhi = static_cast<T*>(it.Bhi) + base;
     T* Blo = static_cast<T*>(it.Blo) + base;
-    for (int f = fg; f < F_pad; f += kPhaseGroups) {
+    for (int f = f_begin; f < f_end; ++f) {
       float2 cv = make_float2(0.f, 0.f);
       if (f < u.nf) {
         const float dh = fwd ? off.f_hi[f] : off.b_hi[f];
@@ -447,7 +448,7 @@ cudaError_t launch_transpose_layers(const float2* W, float2* Wt, int L, int rows
 template <typename T>
 static cudaError_t launch_phases_tc_t(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
                                       const PhaseShape& sh, const Plan* ext, cudaStream_t st) {
-  const int threads = kPhaseModes * kPhaseGroups;
+  const int threads = kPhaseModes;
   const unsigned gx = (4 * sh.max_M + kPhaseModes - 1) / kPhaseModes;
   if (sh.max_I > 1) {
     const dim3 grid(gx, n_entries, (sh.max_I + kIllumGroup - 1) / kIllumGroup);
@@ -462,7 +463,7 @@ static cudaError_t launch_phases_tc_t(const ItemDev& one, const ItemDev* items, 
       phases_illum_kernel<T, false><<<grid, kPhaseModes, smem, st>>>(one, nullptr, d_entries, sh.F_pad);
     return cudaGetLastError();
   }
-  const dim3 grid(gx, n_entries + (ext ? ext->n_exterior : 0));
+  const dim3 grid(gx, n_entries + (ext ? ext->n_exterior : 0), (sh.F_pad + kPhasePlanes - 1) / kPhasePlanes);
   if (items)
     phases_tc_kernel<T, true, false><<<grid, threads, 0, st>>>(one, items, d_entries, sh.F_pad, n_entries, NoExt{});
   else if (ext)

@@ -464,25 +464,37 @@ __global__ void __launch_bounds__(kYregThreads, NGM <= 2 ? 4 : 3)
   const int ns = it.nsplit[f];
   const size_t stride = it.split_stride;
   for (int i0 = 0; i0 < V * Up; i0 += 4 * kYregThreads) {
-    // the first partials of four elements are requested before any is used
-    float2 v[4][2];
+    // four partials of four elements are requested before any is used
+    constexpr int kAhead = 4;
     int off[4];
+    float2 acc[4];
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
       const int i = i0 + h * kYregThreads + threadIdx.x;
       const int vi = i / Up, ui = i < V * Up ? fold_order(i - vi * Up, U, Up) : -1;
       off[h] = ui >= 0 ? vi * U + ui : -1;
+      acc[h] = make_float2(0.f, 0.f);
+    }
+#pragma unroll 1
+    for (int k0 = 0; k0 < ns; k0 += kAhead) {
+      float2 v[4][kAhead];
 #pragma unroll
-      for (int k = 0; k < 2; ++k)
-        v[h][k] = (off[h] >= 0 && k < ns) ? src[(size_t)k * stride + off[h]] : make_float2(0.f, 0.f);
+      for (int k = 0; k < kAhead; ++k)
+#pragma unroll
+        for (int h = 0; h < 4; ++h)
+          v[h][k] = (off[h] >= 0 && k0 + k < ns) ? src[(size_t)(k0 + k) * stride + off[h]] : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        if (k0 == 0) acc[h] = v[h][0];
+        else acc[h] = c_add(acc[h], v[h][0]);
+#pragma unroll
+        for (int k = 1; k < kAhead; ++k) acc[h] = c_add(acc[h], v[h][k]);
+      }
     }
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
       const int i = i0 + h * kYregThreads + threadIdx.x;
-      float2 acc = c_add(v[h][0], v[h][1]);
-      if (off[h] >= 0)
-        for (int k = 2; k < ns; ++k) acc = c_add(acc, src[(size_t)k * stride + off[h]]);
-      if (i < V * Up) srow[i] = acc;
+      if (i < V * Up) srow[i] = acc[h];
     }
   }
   __syncthreads();
