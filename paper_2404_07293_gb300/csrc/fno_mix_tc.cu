@@ -15,14 +15,16 @@
 // into X = X_hi + X_lo (BF16 each), so each mode takes two MMAs into one FP32
 // accumulator: the products keep the weights' BF16 and nearly FP32 spectra.
 //
-// A CTA takes kMixModes = 2 consecutive modes and 128 samples (80 KB of shared memory:
-// two CTAs per SM, one wave at 256 samples). All 256 threads stage the operands straight
+// A CTA takes MODES consecutive modes (2 or 4) and 128 samples with 128 MODES threads (80 KB of shared
+// memory and two CTAs per SM, or 160 KB and one). All threads stage the operands straight
 // from global memory into the 128-byte-swizzled K-major layout the MMA reads (rows of 64
-// BF16 = 128 bytes; 16-byte chunk g of row r at g ^ (r mod 8)); one thread issues the 16
-// MMAs (2 modes x 4 K-steps x 2 halves) into 2 x 64 TMEM columns; the eight warps then
+// BF16 = 128 bytes; 16-byte chunk g of row r at g ^ (r mod 8)); one thread issues the
+// MMAs (MODES x 4 K-steps x 2 halves) into MODES x 64 TMEM columns; the warps then
 // read the accumulators (warp w: TMEM lanes of its quadrant w mod 4 = 32 samples, outputs
-// 16 (w / 4) .. + 15) and write, per sample and output, the two modes as one 8-byte store
-// of the K-major result row.
+// 32 / MODES (w / 4) and on) and write, per sample and output, the modes as one 8- or 16-byte store
+// of the K-major result row. The result rows are 1 KB and more apart, so every store is a part of a 32-byte
+// sector of its own: four modes per CTA halve them, 16.2 -> 12.5 us at 256 samples. One block of samples keeps
+// two modes and twice the CTAs.
 // The single wait (MMA completion) is bounded by a %globaltimer deadline.
 #include "fno_internal.cuh"
 #include "scw_ptx.cuh"
@@ -30,12 +32,12 @@
 namespace scw {
 namespace fno {
 
-constexpr int kMixModes = 2;
 constexpr int kMixRows = 128;
 constexpr int kMaxSplitsUnrolled = 2;  // K-split partials of the spectra loaded in one batch
 constexpr uint32_t kMixABytes = kMixRows * 128u;   // one mode's A (hi or lo): 128 rows x 64 BF16
 constexpr uint32_t kMixBBytes = 64u * 128u;        // one mode's B: 64 rows x 64 BF16
-constexpr uint32_t kMixSmem = 2 * kMixModes * kMixABytes + kMixModes * kMixBBytes + 1024u;
+template <int MODES>
+constexpr uint32_t mix_smem() { return MODES * (2 * kMixABytes + kMixBBytes) + 1024u; }
 
 __device__ __forceinline__ uint32_t swz128(int row, int chunk) {
   return (uint32_t)row * 128u + ((uint32_t)(chunk ^ (row & 7)) << 4);
@@ -44,8 +46,12 @@ __device__ __forceinline__ uint32_t swz128(int row, int chunk) {
 // (a, b) as one BF16 pair: a in the low half (the lower address), b in the high half
 __device__ __forceinline__ uint32_t bf16x2_bits(float a, float b) { return pack_bf16x2(a, b); }
 
-template <bool CONJ>
-__global__ void __launch_bounds__(256, 2) mix_tc_kernel(const float2* __restrict__ X, int splits,
+template <int MODES> struct ModeWords;
+template <> struct ModeWords<2> { typedef uint2 T; };
+template <> struct ModeWords<4> { typedef uint4 T; };
+
+template <bool CONJ, int MODES>
+__global__ void __launch_bounds__(128 * MODES, 4 / MODES) mix_tc_kernel(const float2* __restrict__ X, int splits,
                                                         long long split_stride, long long ld,
                                                         const __nv_bfloat16* __restrict__ R,
                                                         __nv_bfloat16* __restrict__ out, float scale, int B, int Kp,
@@ -55,10 +61,10 @@ __global__ void __launch_bounds__(256, 2) mix_tc_kernel(const float2* __restrict
   __shared__ uint32_t tmem_base_s;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* A_hi = smem;
-  uint8_t* A_lo = smem + kMixModes * kMixABytes;
-  uint8_t* Bop = smem + 2 * kMixModes * kMixABytes;
+  uint8_t* A_lo = smem + MODES * kMixABytes;
+  uint8_t* Bop = smem + 2 * MODES * kMixABytes;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int k0 = blockIdx.x * kMixModes, b0 = blockIdx.y * kMixRows;
+  const int k0 = blockIdx.x * MODES, b0 = blockIdx.y * kMixRows;
   const uint64_t deadline = ptx::globaltimer() + timeout_ns;
 
   if (threadIdx.x == 0) {
@@ -66,7 +72,7 @@ __global__ void __launch_bounds__(256, 2) mix_tc_kernel(const float2* __restrict
     ptx::fence_mbar_init();
   }
   if (warp == 0) {
-    ptx::tmem_alloc(ptx::smem_u32(&tmem_base_s), kMixModes * 64);
+    ptx::tmem_alloc(ptx::smem_u32(&tmem_base_s), MODES * 64);
     ptx::tmem_relinquish();
   }
   pdl_sync();  // the spectra come from the preceding kernels
@@ -75,15 +81,16 @@ __global__ void __launch_bounds__(256, 2) mix_tc_kernel(const float2* __restrict
   // and 4 chunks of B. Every load it needs (R's words, then the first K-split partial of its A
   // chunks) is issued before any value is used: with so little work per CTA the staging is bound
   // by memory round trips.
-  constexpr int kChunks = kMixModes * kMixRows * 8 / 256;  // 8 per thread
+  constexpr int kThreads = 128 * MODES;
+  constexpr int kChunks = MODES * kMixRows * 8 / kThreads;  // 8 per thread
   const uint32_t* R32 = reinterpret_cast<const uint32_t*>(R);
-  constexpr int kBChunks = kMixModes * 64 * 8 / 256;  // 4 per thread
+  constexpr int kBChunks = MODES * 64 * 8 / kThreads;  // 4 per thread
   // B: per mode 64 rows n = 2 p + r (p the output index), chunk g = K values 8 g .. 8 g + 7
   // (inputs 4 g .. 4 g + 3, re and im). R[k][o][i] is stored as BF16 (re, im) pairs.
   uint32_t rv[kBChunks][4];
 #pragma unroll
   for (int jj = 0; jj < kBChunks; ++jj) {
-    const int q = threadIdx.x + 256 * jj;
+    const int q = threadIdx.x + kThreads * jj;
     const int mm = q >> 9, n = (q >> 3) & 63, g = q & 7;
     const int p = n >> 1;
 #pragma unroll
@@ -99,7 +106,7 @@ __global__ void __launch_bounds__(256, 2) mix_tc_kernel(const float2* __restrict
     if (z >= splits) break;  // uniform
 #pragma unroll
     for (int j = 0; j < kChunks; ++j) {
-      const int q = threadIdx.x + 256 * j;
+      const int q = threadIdx.x + kThreads * j;
       const int mm = q >> 10, r = (q >> 3) & (kMixRows - 1), g = q & 7;
       const int b = b0 + r;
       float4 pa = make_float4(0.f, 0.f, 0.f, 0.f), pb = pa;
@@ -121,7 +128,7 @@ __global__ void __launch_bounds__(256, 2) mix_tc_kernel(const float2* __restrict
   for (int z = kMaxSplitsUnrolled; z < splits; ++z) {  // more K-split partials than the unrolled ones (rare)
 #pragma unroll
     for (int j = 0; j < kChunks; ++j) {
-      const int q = threadIdx.x + 256 * j;
+      const int q = threadIdx.x + kThreads * j;
       const int mm = q >> 10, r = (q >> 3) & (kMixRows - 1), g = q & 7;
       const int b = b0 + r;
       if (b < B) {
@@ -135,7 +142,7 @@ __global__ void __launch_bounds__(256, 2) mix_tc_kernel(const float2* __restrict
   }
 #pragma unroll
   for (int j = 0; j < kChunks; ++j) {
-    const int q = threadIdx.x + 256 * j;
+    const int q = threadIdx.x + kThreads * j;
     const int mm = q >> 10, r = (q >> 3) & (kMixRows - 1), g = q & 7;
     const float v[8] = {va[j].x, va[j].y, va[j].z, va[j].w, vb[j].x, vb[j].y, vb[j].z, vb[j].w};
     uint32_t h[4], l[4];
@@ -151,7 +158,7 @@ __global__ void __launch_bounds__(256, 2) mix_tc_kernel(const float2* __restrict
   }
 #pragma unroll
   for (int jj = 0; jj < kBChunks; ++jj) {
-    const int q = threadIdx.x + 256 * jj;
+    const int q = threadIdx.x + kThreads * jj;
     const int mm = q >> 9, n = (q >> 3) & 63, g = q & 7;
     const int rr = n & 1;
     uint32_t w[4];
@@ -180,7 +187,7 @@ __global__ void __launch_bounds__(256, 2) mix_tc_kernel(const float2* __restrict
   if (threadIdx.x == 0) {
     constexpr uint32_t idesc = ptx::idesc_f16(true, 128, 64);
 #pragma unroll
-    for (int mm = 0; mm < kMixModes; ++mm) {
+    for (int mm = 0; mm < MODES; ++mm) {
       const uint64_t dh = ptx::sw128_desc(ptx::smem_u32(A_hi + mm * kMixABytes));
       const uint64_t dl = ptx::sw128_desc(ptx::smem_u32(A_lo + mm * kMixABytes));
       const uint64_t db = ptx::sw128_desc(ptx::smem_u32(Bop + mm * kMixBBytes));
@@ -201,25 +208,26 @@ __global__ void __launch_bounds__(256, 2) mix_tc_kernel(const float2* __restrict
       atomicOr(err, DEV_ERR_TIMEOUT_DRAIN);
   } else {
     ptx::tc_fence_after();
-    const int quad = warp & 3, half = warp >> 2;
+    const int quad = warp & 3, o_begin = (warp >> 2) * (C / MODES);
     const int b = b0 + quad * 32 + lane;
     const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
 #pragma unroll 1
-    for (int o0 = 16 * half; o0 < 16 * half + 16; o0 += 4) {
-      uint32_t v[kMixModes][8];  // mode mm: outputs o0 .. o0 + 3, (re, im) each
+    for (int o0 = o_begin; o0 < o_begin + C / MODES; o0 += 4) {
+      uint32_t v[MODES][8];  // mode mm: outputs o0 .. o0 + 3, (re, im) each
 #pragma unroll
-      for (int mm = 0; mm < kMixModes; ++mm) ptx::tmem_ld_x8(lane_base + (uint32_t)(mm * 64 + 2 * o0), v[mm]);
+      for (int mm = 0; mm < MODES; ++mm) ptx::tmem_ld_x8(lane_base + (uint32_t)(mm * 64 + 2 * o0), v[mm]);
       ptx::tmem_wait_ld();
       if (b < B) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          uint32_t w[kMixModes];
+          alignas(16) uint32_t w[MODES];
 #pragma unroll
-          for (int mm = 0; mm < kMixModes; ++mm)
+          for (int mm = 0; mm < MODES; ++mm)
             w[mm] = bf16x2_bits(scale * __uint_as_float(v[mm][2 * e]), scale * __uint_as_float(v[mm][2 * e + 1]));
-          // row (b, o) of the K-major result, modes k0, k0 + 1 (k0 even: 8-byte aligned)
-          *reinterpret_cast<uint2*>(reinterpret_cast<uint32_t*>(out) + ((size_t)b * C + o0 + e) * (Kp / 2) + k0) =
-              make_uint2(w[0], w[1]);
+          // row (b, o) of the K-major result, modes k0 .. k0 + MODES - 1 (k0 and Kp / 2 are multiples of MODES)
+          *reinterpret_cast<typename ModeWords<MODES>::T*>(reinterpret_cast<uint32_t*>(out) +
+                                                           ((size_t)b * C + o0 + e) * (Kp / 2) + k0) =
+              *reinterpret_cast<typename ModeWords<MODES>::T*>(w);
         }
       }
     }
@@ -228,7 +236,7 @@ __global__ void __launch_bounds__(256, 2) mix_tc_kernel(const float2* __restrict
   __syncthreads();
   if (warp == 0) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem, kMixModes * 64);
+    ptx::tmem_dealloc(tmem, MODES * 64);
   }
 }
 
@@ -427,14 +435,17 @@ cudaError_t launch_mix_dr_tc(const float2* G, const float2* V, int splits, long 
 cudaError_t launch_mix_tc(bool conj, const float2* X, int splits, long long split_stride, long long ld,
                           const __nv_bfloat16* R, __nv_bfloat16* out, float scale, int B, int m, int Kp, int* err,
                           uint64_t timeout_ns, cudaStream_t st) {
-  if ((m * m) % kMixModes || Kp % 8 || (ld % 2) || (split_stride % 2)) return cudaErrorInvalidValue;
-  const void* fn = conj ? reinterpret_cast<const void*>(mix_tc_kernel<true>)
-                        : reinterpret_cast<const void*>(mix_tc_kernel<false>);
-  cudaError_t e = allow_max_smem(fn);
-  if (e != cudaSuccess) return e;
-  const dim3 grid(m * m / kMixModes, (B + kMixRows - 1) / kMixRows);
-  return launch_pdl(conj ? mix_tc_kernel<true> : mix_tc_kernel<false>, grid, dim3(256), kMixSmem, st, X, splits,
-                    split_stride, ld, R, out, scale, B, Kp, err, timeout_ns);
+  if ((m * m) % 2 || Kp % 8 || (ld % 2) || (split_stride % 2)) return cudaErrorInvalidValue;
+  const int blocks = (B + kMixRows - 1) / kMixRows;
+  auto run = [&](auto kernel, int modes, uint32_t smem) -> cudaError_t {
+    cudaError_t e = allow_max_smem(reinterpret_cast<const void*>(kernel));
+    if (e != cudaSuccess) return e;
+    return launch_pdl(kernel, dim3(m * m / modes, blocks), dim3(128 * modes), smem, st, X, splits, split_stride, ld, R, out,
+                      scale, B, Kp, err, timeout_ns);
+  };
+  if ((m * m) % 4 == 0 && blocks > 1)
+    return conj ? run(mix_tc_kernel<true, 4>, 4, mix_smem<4>()) : run(mix_tc_kernel<false, 4>, 4, mix_smem<4>());
+  return conj ? run(mix_tc_kernel<true, 2>, 2, mix_smem<2>()) : run(mix_tc_kernel<false, 2>, 2, mix_smem<2>());
 }
 
 }  // namespace fno

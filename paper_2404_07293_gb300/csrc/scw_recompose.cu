@@ -818,7 +818,7 @@ cudaError_t launch_recompose_fused(const ItemDev& one, const ItemDev* items, con
     cudaError_t e = allow_max_smem(reinterpret_cast<const void*>(recompose_fused_kernel<B, T, G>));              \
     if (e != cudaSuccess) return e;                                                                              \
     return launch_pdl(recompose_fused_kernel<B, T, G>, dim3((unsigned)grid), dim3(kYregThreads), smem, st, one,   \
-                      items, d_entries, (int)whole, ysplit, out_one, d_outs);                                                                           \
+                      items, d_entries, (int)whole, ysplit, out_one, d_outs);                                    \
   }()
 #define SCW_FG(B, T) (ngm == 2 ? SCW_FU(B, T, 2) : ngm == 3 ? SCW_FU(B, T, 3) : SCW_FU(B, T, 6))
   if (items) return tiled ? SCW_FG(true, true) : SCW_FG(true, false);
