@@ -57,7 +57,7 @@ struct scw_fno_s {
   int* d_err = nullptr;
   uint64_t timeout_ns = 2000000000ull;
 
-  CUtensorMap map_Vcf[9], map_dZcf[2], map_D[kDftTileCount], map_E, map_Wh, map_GVh;
+  CUtensorMap map_Vcf[9], map_dZcf[2], map_D[kDftTileCount], map_E, map_Wh[3], map_GVh[3];
   // 1x1-convolution operands: channel-first activations read MN-major (3D maps), W and W^T
   CUtensorMap map_Vx[8], map_dZx[2], map_W[8], map_WT[8];
 
@@ -200,7 +200,7 @@ static cudaError_t refresh_wt(scw_fno_s* f, cudaStream_t st) {
 // ---------------------------------------------------------------- forward ---
 template <typename T>
 static scw_status forward(scw_fno_s* f, const float2* n, int B, bool keep_z, cudaStream_t st) {
-  const int BC = B * C;
+  const int BC = B * C, bn = layer_tile(f->P, BC);
   // BF16 mode reads the layer inputs channel-first only; the FP32 (SIMT) mode also reads them
   // channel-last
   FNO_TRY(launch_ok(f, launch_lift<T>(n, at<T>(f->wcopy, f->off_P), static_cast<T*>(f->Vcf[0]),
@@ -248,7 +248,7 @@ static scw_status forward(scw_fno_s* f, const float2* n, int B, bool keep_z, cud
     eb.out_cf = l < f->L - 1 ? f->Vcf[l + 1] : nullptr;
     eb.out_cl = (!f->bf16 || l == f->L - 1) ? f->Vcl[l + 1] : nullptr;
     eb.gelu = l < f->L - 1 ? 1 : 0;
-    e = f->bf16 ? launch_gemm_tc(EPI_LAYER_FWD, 256, f->map_E, f->map_Wh, f->map_Vx[l], f->map_W[l], eb, f->P, BC,
+    e = f->bf16 ? launch_gemm_tc(EPI_LAYER_FWD, bn, f->map_E, f->map_Wh[bn / 128], f->map_Vx[l], f->map_W[l], eb, f->P, BC,
                                  f->Kp, 1, f->d_err, f->timeout_ns, st)
                 : launch_gemm_simt(EPI_LAYER_FWD, static_cast<const float*>(f->E), f->Kp,
                                    static_cast<const float*>(f->Wh), f->Kp, eb, f->P, BC, f->Kp, 1, st);
@@ -298,7 +298,7 @@ static scw_status forward_backward(scw_fno_s* f, const float2* n, const float2* 
   if (e == cudaSuccess) e = cudaMemsetAsync(f->loss_d, 0, 4 * sizeof(float), st);
   if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync");
   FNO_TRY(forward<T>(f, n, B, true, st));
-  const int BC = B * C, P = f->P, nblk = f->nblk;
+  const int BC = B * C, P = f->P, nblk = f->nblk, bn = layer_tile(P, BC);
   std::vector<RedSeg> segs;
   FNO_TRY(launch_ok(f, launch_target_norm(target, f->part_tn, B, P, st), "target norm"));
   FNO_TRY(launch_ok(f, launch_project_train<T>(static_cast<const T*>(f->Vcl[f->L]), target, at<T>(f->wcopy, f->off_Q),
@@ -385,7 +385,7 @@ static scw_status forward_backward(scw_fno_s* f, const float2* n, const float2* 
     // dV_0 is consumed by the lift backward only, in the layout it reads
     eb.out_cf = l > 0 || lift_cf ? f->dZcf[1 - cur] : nullptr;
     eb.out_cl = (!f->bf16 || (l == 0 && !lift_cf)) ? f->dZcl[1 - cur] : nullptr;
-    e = f->bf16 ? launch_gemm_tc(EPI_LAYER_BWD, 256, f->map_E, f->map_GVh, f->map_dZx[cur], f->map_WT[l], eb, P, BC,
+    e = f->bf16 ? launch_gemm_tc(EPI_LAYER_BWD, bn, f->map_E, f->map_GVh[bn / 128], f->map_dZx[cur], f->map_WT[l], eb, P, BC,
                                  f->Kp, 1, f->d_err, f->timeout_ns, st)
                 : launch_gemm_simt(EPI_LAYER_BWD, static_cast<const float*>(f->E), f->Kp,
                                    static_cast<const float*>(f->GVh), f->Kp, eb, P, BC, f->Kp, 1, st);
@@ -581,8 +581,10 @@ scw_status scw_surrogate_create(const scw_fno_desc* d, scw_fno_t* out) {
     for (int i = 0; i < kDftTileCount && s == SCW_OK; ++i)
       s = make_map_bf16(&f->map_D[i], f->D, f->P, 2 * f->n_ind, f->P, kDftTiles[i]);
     if (s == SCW_OK) s = make_map_bf16(&f->map_E, f->E, f->Kp, f->P, f->Kp, 128);
-    if (s == SCW_OK) s = make_map_bf16(&f->map_Wh, f->Wh, f->Kp, BCm, f->Kp, 256);
-    if (s == SCW_OK) s = make_map_bf16(&f->map_GVh, f->GVh, f->Kp, BCm, f->Kp, 256);
+    for (int i = 0; i < 3 && s == SCW_OK; ++i) {
+      s = make_map_bf16(&f->map_Wh[i], f->Wh, f->Kp, BCm, f->Kp, kLayerTiles[i]);
+      if (s == SCW_OK) s = make_map_bf16(&f->map_GVh[i], f->GVh, f->Kp, BCm, f->Kp, kLayerTiles[i]);
+    }
     for (int l = 0; l <= f->L && s == SCW_OK; ++l) s = make_map_bf16(&f->map_Vcf[l], f->Vcf[l], f->P, BCm, f->P, 128);
     for (int i = 0; i < 2 && s == SCW_OK; ++i) s = make_map_bf16(&f->map_dZcf[i], f->dZcf[i], f->P, BCm, f->P, 128);
     for (int l = 0; l < f->L && s == SCW_OK; ++l) {

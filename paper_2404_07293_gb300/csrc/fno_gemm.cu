@@ -230,12 +230,12 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_tc_kernel(const __grid_c
   }
 }
 
-// Persistent form of the layer products (EPI_LAYER_FWD / EPI_LAYER_BWD, BN = 256): one
+// Persistent form of the layer products (EPI_LAYER_FWD / EPI_LAYER_BWD) and of the field product: one
 // CTA per SM walks the output tiles t = blockIdx.x, blockIdx.x + gridDim.x, ... (pixel
 // tile fastest, so CTAs in flight share their Wh / GVh tile through L2). Four operand
-// stages; two 256-column TMEM accumulators, so the epilogue of one tile runs while the
+// stages; two TMEM accumulators of BN columns, so the epilogue of one tile runs while the
 // MMAs of the next one are issued (acc_full / acc_empty barriers, as in the contraction).
-// Twelve epilogue warps (three per TMEM lane quadrant) share the 8 column chunks.
+// Twelve epilogue warps (three per TMEM lane quadrant) share the BN / 32 column chunks. BN: layer_tile.
 constexpr int kLayerStages = 4;
 constexpr uint32_t kLayerStage = GemmCfg<256>::STAGE;
 constexpr uint32_t kLayerSmem = kLayerStages * kLayerStage + 1024u;
@@ -287,7 +287,7 @@ __device__ __forceinline__ void epilogue_bwd_z(const EpiArgs& a, int row, int co
   }
 }
 
-template <int EPI>
+template <int EPI, int BN>
 __global__ void __launch_bounds__(kLayerThreads, 1) gemm_layer_persistent(const __grid_constant__ CUtensorMap mA,
                                                                          const __grid_constant__ CUtensorMap mB,
                                                                          const __grid_constant__ CUtensorMap mA2,
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(kLayerThreads, 1) gemm_layer_persistent(const 
                                                                          const __grid_constant__ EpiArgs ea, int K,
                                                                          int m_tiles, int n_tiles, int* err,
                                                                          uint64_t timeout_ns) {
-  constexpr int BN = 256;
+  static_assert(BN == 64 || BN == 128 || BN == 256, "whole samples, and accumulators of a power of two columns");
   constexpr int STAGES = kLayerStages;
   constexpr uint32_t A_BYTES = GemmCfg<256>::A_BYTES;
   extern __shared__ uint8_t smem_raw[];
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(kLayerThreads, 1) gemm_layer_persistent(const 
         const uint32_t fb = ptx::smem_u32(&full_bar[st]);
         const uint32_t sa = ptx::smem_u32(smem + (size_t)st * kLayerStage);
         if (i < nkb) {
-          ptx::mbar_arrive_expect_tx(fb, kLayerStage, leader);
+          ptx::mbar_arrive_expect_tx(fb, A_BYTES + BN * 128u, leader);
           ptx::tma_load_2d(sa, &mA, i * 64, m0, fb, leader);
           ptx::tma_load_2d(sa + A_BYTES, &mB, i * 64, n0, fb, leader);
         } else {
@@ -596,19 +596,55 @@ static cudaError_t launch_tc_t(const CUtensorMap& mA, const CUtensorMap& mB, con
                     err, timeout_ns);
 }
 
-template <int EPI>
+static int device_sms() {
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
+// Waves of tiles times the time of one, which is about BN columns and a fixed part as long as 64 of them (the
+// operand pipeline's latency and the row tile's load). Inference on 64 x 64 pixels, us at tiles of 64, 128 and
+// 256 columns: 5 samples 88.8, 92.9, 96.4; 10 samples 100.2, 95.3, 103.2; 20 samples 115.0, 109.8, 109.5; 48
+// samples 161, 140, 147; 64 samples 179, 160, 155; 256 samples 483, 377, 335.
+constexpr int kLayerTileCost = 64;
+
+template <int EPI, int BN>
 static cudaError_t launch_layer_persistent(const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mA2,
                                            const CUtensorMap& mW, const EpiArgs& ea, int M, int N, int K, int* err,
                                            uint64_t timeout_ns, cudaStream_t st) {
-  const void* fn = reinterpret_cast<const void*>(gemm_layer_persistent<EPI>);
+  const void* fn = reinterpret_cast<const void*>(gemm_layer_persistent<EPI, BN>);
   cudaError_t e = allow_max_smem(fn);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int m_tiles = (M + 127) / 128, n_tiles = (N + 255) / 256;
-  const int grid = std::max(1, std::min(m_tiles * n_tiles, sms));
-  return launch_pdl(gemm_layer_persistent<EPI>, dim3(grid), dim3(kLayerThreads), kLayerSmem, st, mA, mB, mA2, mW, ea, K,
+  const int m_tiles = (M + 127) / 128, n_tiles = (N + BN - 1) / BN;
+  const int grid = std::max(1, std::min(m_tiles * n_tiles, device_sms()));
+  return launch_pdl(gemm_layer_persistent<EPI, BN>, dim3(grid), dim3(kLayerThreads), kLayerSmem, st, mA, mB, mA2, mW, ea, K,
                     m_tiles, n_tiles, err, timeout_ns);
+}
+
+template <int EPI>
+static cudaError_t launch_layer(int BN, const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mA2,
+                                const CUtensorMap& mW, const EpiArgs& ea, int M, int N, int K, int* err,
+                                uint64_t timeout_ns, cudaStream_t st) {
+  switch (BN) {
+    case 64: return launch_layer_persistent<EPI, 64>(mA, mB, mA2, mW, ea, M, N, K, err, timeout_ns, st);
+    case 128: return launch_layer_persistent<EPI, 128>(mA, mB, mA2, mW, ea, M, N, K, err, timeout_ns, st);
+    case 256: return launch_layer_persistent<EPI, 256>(mA, mB, mA2, mW, ea, M, N, K, err, timeout_ns, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+int layer_tile(int M, int N) {
+  const long long sms = device_sms(), m_tiles = (M + 127) / 128;
+  int best = 256;
+  long long best_cost = 0;
+  for (int bn = 256; bn >= 64; bn /= 2) {
+    const long long tiles = m_tiles * ((N + bn - 1) / bn), cost = (tiles + sms - 1) / sms * (bn + kLayerTileCost);
+    if (bn == 256 || cost < best_cost) {
+      best = bn;
+      best_cost = cost;
+    }
+  }
+  return best;
 }
 
 template <int EPI>
@@ -630,16 +666,16 @@ cudaError_t launch_gemm_tc(int epi, int BN, const CUtensorMap& mA, const CUtenso
   if (K % 64 != 0 || splits < 1) return cudaErrorInvalidValue;
   const bool layer = epi == EPI_LAYER_FWD || epi == EPI_LAYER_BWD;
   // the 1x1 segment shares the accumulator: the DFT part must come pre-scaled (alpha 1)
-  if (layer && (splits != 1 || BN != 256 || ea.alpha != 1.0f)) return cudaErrorInvalidValue;
+  if (layer && (splits != 1 || ea.alpha != 1.0f)) return cudaErrorInvalidValue;
   switch (epi) {
     case EPI_LAYER_FWD:
-      return launch_layer_persistent<EPI_LAYER_FWD>(mA, mB, mA2, mW, ea, M, N, K, err, timeout_ns, st);
+      return launch_layer<EPI_LAYER_FWD>(BN, mA, mB, mA2, mW, ea, M, N, K, err, timeout_ns, st);
     case EPI_LAYER_BWD:
-      return launch_layer_persistent<EPI_LAYER_BWD>(mA, mB, mA2, mW, ea, M, N, K, err, timeout_ns, st);
+      return launch_layer<EPI_LAYER_BWD>(BN, mA, mB, mA2, mW, ea, M, N, K, err, timeout_ns, st);
     case EPI_FIELD:
       if (splits != 1) return cudaErrorInvalidValue;
       // BN 256: the persistent form (epilogue of one tile overlapping the next tile's MMAs)
-      return BN == 256 ? launch_layer_persistent<EPI_FIELD>(mA, mB, mA2, mW, ea, M, N, K, err, timeout_ns, st)
+      return BN == 256 ? launch_layer_persistent<EPI_FIELD, 256>(mA, mB, mA2, mW, ea, M, N, K, err, timeout_ns, st)
                        : launch_tc_bn<EPI_FIELD>(BN, mA, mB, mA2, mW, ea, M, N, K, 1, err, timeout_ns, st);
     default: return cudaErrorInvalidValue;
   }

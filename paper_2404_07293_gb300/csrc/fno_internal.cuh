@@ -324,6 +324,9 @@ __device__ __forceinline__ void epilogue(const EpiArgs& a, const float* w_s, con
 // [C][C] with box {32, 32} and 64-byte swizzle); they run on the tensor cores as one extra
 // K = 32 segment per sample of the tile, into that sample's 32 columns, kSeg2Samples samples
 // per operand stage.
+// Tile width of a layer product (64, 128 or 256 columns; the box of mB) for M pixels and N = B C columns.
+int layer_tile(int M, int N);
+constexpr int kLayerTiles[3] = {64, 128, 256};
 cudaError_t launch_gemm_tc(int epi, int BN, const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mA2,
                            const CUtensorMap& mW, const EpiArgs& ea, int M, int N, int K, int splits, int* err,
                            uint64_t timeout_ns, cudaStream_t st);
