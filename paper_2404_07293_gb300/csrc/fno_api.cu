@@ -224,7 +224,7 @@ static scw_status forward(scw_fno_s* f, const float2* n, int B, bool keep_z, cud
                                             f->timeout_ns, st)
                             : launch_gemm_simt(EPI_MODES, static_cast<const float*>(f->Vcf[l]), f->P,
                                                static_cast<const float*>(f->D), f->P, ea, BC, Kd, f->P, ks, st);
-    FNO_TRY(launch_ok(f, e, "truncated DFT", CAT_DFT, 2.0 * BC * f->Kc * f->P));
+    FNO_TRY(launch_ok(f, e, "truncated DFT", CAT_DFT, 2.0 * BC * Kd * f->P));
     // Wh carries the inverse transform's 1/N^2 so that the 1x1 convolution can share its accumulator
     if constexpr (std::is_same<T, __nv_bfloat16>::value)
       e = launch_mix_tc(false, reinterpret_cast<const float2*>(f->Vh[l]), ks, vstride, ld, at<T>(f->wcopy, f->off_R[l]),
@@ -340,11 +340,11 @@ static scw_status forward_backward(scw_fno_s* f, const float2* n, const float2* 
     if (f->bf16) {
       e = launch_dft_tc(f->map_dZcf[cur], f->map_D, &f->map_Vcf[l], ea, &ew, BC, Kd, P, f->d_err, f->timeout_ns, st);
       FNO_TRY(launch_ok(f, e, "truncated DFT of dZ and weight gradient", CAT_DFT,
-                        2.0 * BC * f->Kc * P + 2.0 * BC * C * P));
+                        2.0 * BC * Kd * P + 2.0 * BC * C * P));
     } else {
       e = launch_gemm_simt(EPI_MODES, static_cast<const float*>(f->dZcf[cur]), P, static_cast<const float*>(f->D), P,
                            ea, BC, Kd, P, ks, st);
-      FNO_TRY(launch_ok(f, e, "truncated DFT of dZ", CAT_DFT, 2.0 * BC * f->Kc * P));
+      FNO_TRY(launch_ok(f, e, "truncated DFT of dZ", CAT_DFT, 2.0 * BC * Kd * P));
       e = launch_gemm_simt(EPI_DW, static_cast<const float*>(f->dZcf[cur]), P, static_cast<const float*>(f->Vcf[l]), P,
                            ew, groups * 128, groups * 128, P, kw, st);
       FNO_TRY(launch_ok(f, e, "weight gradient", CAT_DW, 2.0 * BC * C * P));

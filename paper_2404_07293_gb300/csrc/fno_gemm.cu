@@ -8,9 +8,9 @@
 // tensor memory; eight epilogue warps read it back with tcgen05.ld (one TMEM lane
 // per thread = one row of D; two warps per 32-lane quadrant split the columns)
 // and apply the epilogue 32 columns at a time.
-//   warp 0 lane 0   TMA producer (full/empty mbarriers per stage)
-//   warp 1 lane 0   MMA issuer; commits each stage back to the producer
-//   warps 2-9       epilogue
+//   warp 0      TMA producer (full/empty mbarriers per stage)
+//   warp 1      MMA issuer; commits each stage back to the producer
+//   warps 2-9   epilogue
 // The layer products add the 1x1 convolution as a second K segment: for each
 // sample s of the tile, D[:, 32 s .. 32 s + 32) += X_s W^T (X_s = that sample's
 // activations at the tile's 128 pixels, K = 32 channels, N = 32 MMAs into the
@@ -50,10 +50,9 @@ struct GemmCfg {
   static constexpr uint32_t A_BYTES = 128u * 128u;            // 128 rows x 64 bf16
   static constexpr uint32_t B_BYTES = (uint32_t)BN * 128u;     // BN rows x 64 bf16
   static constexpr uint32_t STAGE = A_BYTES + B_BYTES;
-  static constexpr int ST_RAW = (int)(100u * 1024u / STAGE);   // two CTAs per SM
-  static constexpr int STAGES = ST_RAW < 2 ? 2 : (ST_RAW > 6 ? 6 : ST_RAW);
+  static constexpr int STAGES = (int)(100u * 1024u / STAGE);   // two CTAs per SM
   static constexpr uint32_t SMEM = STAGES * STAGE + 1024u;
-  static constexpr uint32_t TMEM_COLS = BN < 32 ? 32u : (uint32_t)BN;
+  static constexpr uint32_t TMEM_COLS = (uint32_t)BN;
 };
 
 constexpr int kGemmThreads = 320;
@@ -652,10 +651,8 @@ static cudaError_t launch_tc_bn(int BN, const CUtensorMap& mA, const CUtensorMap
                                 const CUtensorMap& mW, const EpiArgs& ea, int M, int N, int K, int splits, int* err,
                                 uint64_t timeout_ns, cudaStream_t st) {
   switch (BN) {
-    case 32: return launch_tc_t<32, EPI>(mA, mB, mA2, mW, ea, M, N, K, splits, err, timeout_ns, st);
     case 64: return launch_tc_t<64, EPI>(mA, mB, mA2, mW, ea, M, N, K, splits, err, timeout_ns, st);
     case 128: return launch_tc_t<128, EPI>(mA, mB, mA2, mW, ea, M, N, K, splits, err, timeout_ns, st);
-    case 256: return launch_tc_t<256, EPI>(mA, mB, mA2, mW, ea, M, N, K, splits, err, timeout_ns, st);
     default: return cudaErrorInvalidValue;
   }
 }

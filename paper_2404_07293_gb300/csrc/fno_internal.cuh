@@ -316,17 +316,17 @@ __device__ __forceinline__ void epilogue(const EpiArgs& a, const float* w_s, con
 }
 
 // ---- launchers ---------------------------------------------------------------------------
+// Tile width of a layer product (64, 128 or 256 columns; the box of mB) for M pixels and N = B C columns.
+int layer_tile(int M, int N);
+constexpr int kLayerTiles[3] = {64, 128, 256};
 // Tensor-core GEMM D = A B^T over K (bf16, K-major, TMA maps with 128-byte swizzle and
-// a 64-element inner box): A rows in boxes of 128, B rows in boxes of BN (32..256).
+// a 64-element inner box): A rows in boxes of 128, B rows in boxes of BN (64, 128 or 256).
 // grid = (ceil(N/BN), ceil(M/128), splits). Each split covers kper 64-wide K blocks.
 // EPI_LAYER_*: mA2 / mW are the 1x1-convolution operands (channel-first activations [B][C][P]
 // as a 3D map with box {64, 32, kSeg2Samples} and 128-byte swizzle, read MN-major; W or W^T
 // [C][C] with box {32, 32} and 64-byte swizzle); they run on the tensor cores as one extra
 // K = 32 segment per sample of the tile, into that sample's 32 columns, kSeg2Samples samples
 // per operand stage.
-// Tile width of a layer product (64, 128 or 256 columns; the box of mB) for M pixels and N = B C columns.
-int layer_tile(int M, int N);
-constexpr int kLayerTiles[3] = {64, 128, 256};
 cudaError_t launch_gemm_tc(int epi, int BN, const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mA2,
                            const CUtensorMap& mW, const EpiArgs& ea, int M, int N, int K, int splits, int* err,
                            uint64_t timeout_ns, cudaStream_t st);
