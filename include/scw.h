@@ -88,7 +88,9 @@ enum {
                              SCW_ERR_BOUNDS. The bulk copies of the tensor-core contraction
                              are driven by a task table built on the host: plan creation
                              checks every task's W, B and partial-spectrum ranges against
-                             their allocations and fails with SCW_ERR_BOUNDS. Results are
+                             their allocations and fails with SCW_ERR_BOUNDS. Where step (c)
+                             is one kernel, the plan runs it and then the x-pass and the y-pass
+                             over the same field, so that every form is checked. Results are
                              the same as without the flag; the checks cost a compare per
                              access or per loop                                         */
 };

@@ -575,6 +575,7 @@ struct scw_plan_s {
   int n_plane_entries = 0;
   int n_long_entries = 0;
   bool tiled = false;  // some item stores periodic tiles
+  bool checked = false;  // some item has SCW_FLAG_DEBUG_BOUNDS
   int max_twy = 0;     // largest y fold-twiddle table (complex elements)
   int inject_stall = 0;            // scw_plan_inject_stall (tests of the timeout path)
   unsigned long long* d_trace = nullptr;  // kernel trace stamps (scw_plan_enable_trace), or null
@@ -789,12 +790,15 @@ static scw_status enqueue_synthesis(scw_plan_t P, float2* out_one, cudaStream_t 
   mark(P, 2, st, marks);
   cudaError_t e;
   if (P->fused_smem) {
-    mark(P, 3, st, marks);  // one kernel: its time is the y-pass's
+    if (!P->checked) mark(P, 3, st, marks);  // one kernel: its time is the y-pass's
     e = launch_recompose_fused(one, items, P->d_plane_entries, P->n_plane_entries, P->max_Vp, P->fused_smem, P->tiled,
-                               out_one, P->d_outs, st);
+                               P->checked, out_one, P->d_outs, st);
     if (e != cudaSuccess) return cuda_error(e, "recompose launch");
-    mark(P, 4, st, marks);
     ++n;
+  }
+  // index-check plans run the two kernels as well, over the same field: the indices of every form are checked
+  if (P->fused_smem && !P->checked) {
+    mark(P, 4, st, marks);
     if (marks && P->timing && P->tev_used + kMarks <= P->tev.size()) P->tev_used += kMarks;
     return SCW_OK;
   }
@@ -1007,7 +1011,6 @@ static size_t fuse_recompose(const scw_plan_t P, int n_planes) {
   if (3 * n_planes < kFuseTiles) return 0;
   size_t smem = 0;
   for (const Plan* p : P->items) {
-    if (p->flags & SCW_FLAG_DEBUG_BOUNDS) return 0;  // the two kernels carry the index checks
     const size_t b = fused_recompose_smem(p->U, p->V, p->Fx, p->Fy);
     if (b == 0) return 0;
     smem = std::max(smem, b);
@@ -1037,6 +1040,7 @@ static scw_status finish_plan(scw_plan_t P, const std::vector<int>& user_ks, boo
     P->max_Vp = std::max(P->max_Vp, p->item.Vp);
     P->rec_smem = std::max(P->rec_smem, recompose_smem_bytes(p->V, p->item.Up, p->item.Vp));
     P->tiled = P->tiled || p->tiles_x > 1 || p->tiles_y > 1;
+    P->checked = P->checked || (p->flags & SCW_FLAG_DEBUG_BOUNDS) != 0;
     P->max_twy = std::max(P->max_twy, (p->Fy / 8) * p->item.Vp);
   }
   // plane entries of items with long y folds first: they run the shared-memory y-pass

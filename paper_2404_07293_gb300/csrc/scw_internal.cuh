@@ -281,11 +281,11 @@ cudaError_t launch_ypass(const ItemDev& one, const ItemDev* items, const int2* d
                          int max_Qx, int max_Vp, int max_twy, bool tiled, float2* out_one, float2* const* d_outs,
                          cudaStream_t st, int* launches);
 // Both directions in one kernel. fused_recompose_smem: its shared memory for an item, 0 where the item does
-// not fit it; launch: smem is the largest of the items.
+// not fit it; launch: smem is the largest of the items; checked: the form with index checks.
 size_t fused_recompose_smem(int U, int V, int Fx, int Fy);
 cudaError_t launch_recompose_fused(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
-                                   int max_Vp, size_t smem, bool tiled, float2* out_one, float2* const* d_outs,
-                                   cudaStream_t st);
+                                   int max_Vp, size_t smem, bool tiled, bool checked, float2* out_one,
+                                   float2* const* d_outs, cudaStream_t st);
 cudaError_t launch_recompose(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries, int max_Qx,
                              size_t smem, const float2* S_override, const int* nsplit_override, float2* out_one,
                              float2* const* d_outs, cudaStream_t st);

@@ -439,7 +439,9 @@ __device__ __forceinline__ void fused_y(const ItemDev& it, const float2* rows, c
   }
 }
 
-template <bool BATCH, bool TILED, int NGM>
+// CHK: the index checks of SCW_FLAG_DEBUG_BOUNDS plans, a form of its own: as run-time branches they cost other
+// plans up to 10 % (9 x 9 orders, 64 planes of 128 x 128: 18.7 -> 20.6 us).
+template <bool BATCH, bool TILED, int NGM, bool CHK>
 __global__ void __launch_bounds__(kYregThreads, NGM <= 2 ? 4 : 3)
     recompose_fused_kernel(const __grid_constant__ ItemDev one, const ItemDev* __restrict__ items,
                            const int2* __restrict__ entries, int whole, int ysplit_rest, float2* out_one,
@@ -457,11 +459,15 @@ __global__ void __launch_bounds__(kYregThreads, NGM <= 2 ? 4 : 3)
   float4* twy = fu_s4 + (size_t)V * Fx / 2;
   float2* twx = reinterpret_cast<float2*>(twy + (size_t)Qy * Vp / 2);
   float2* srow = twx + (size_t)Up * Qx;
-  for (int i = threadIdx.x; i < Qy * Vp / 2; i += kYregThreads) twy[i] = __ldg(reinterpret_cast<const float4*>(it.twy) + i);
-  for (int i = threadIdx.x; i < Up * Qx; i += kYregThreads) twx[i] = __ldg(it.twx + i);
+  for (int i = threadIdx.x; i < Qy * Vp / 2; i += kYregThreads)
+    twy[i] = !CHK || in_bounds(it, BND_TWY, 2 * (size_t)i + 1) ? __ldg(reinterpret_cast<const float4*>(it.twy) + i)
+                                                               : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int i = threadIdx.x; i < Up * Qx; i += kYregThreads)
+    twx[i] = !CHK || in_bounds(it, BND_TWX, i) ? __ldg(it.twx + i) : make_float2(0.f, 0.f);
   ptx::griddep_wait();  // the partial spectra come from the preceding contraction
   trace_begin(one.trace, TRACE_YPASS);
-  const float2* src = it.S_part + (size_t)f * 3 * M + (size_t)c * M;
+  const size_t sbase = (size_t)f * 3 * M + (size_t)c * M;
+  const float2* src = it.S_part + sbase;
   const int ns = it.nsplit[f];
   const size_t stride = it.split_stride;
   for (int i0 = 0; i0 < V * Up; i0 += 4 * kYregThreads) {
@@ -475,6 +481,8 @@ __global__ void __launch_bounds__(kYregThreads, NGM <= 2 ? 4 : 3)
       const int i = i0 + h * kYregThreads + threadIdx.x;
       const int vi = i / Up, ui = i < V * Up ? fold_order(i - vi * Up, U, Up) : -1;
       off[h] = ui >= 0 ? vi * U + ui : -1;
+      // the element's last partial has the largest index
+      if (CHK && off[h] >= 0 && !in_bounds(it, BND_S_PART, sbase + (size_t)(ns - 1) * stride + off[h])) off[h] = -1;
       acc[h] = make_float2(0.f, 0.f);
     }
 #pragma unroll 1
@@ -792,8 +800,8 @@ size_t fused_recompose_smem(int U, int V, int Fx, int Fy) {
 }
 
 cudaError_t launch_recompose_fused(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
-                                   int max_Vp, size_t smem, bool tiled, float2* out_one, float2* const* d_outs,
-                                   cudaStream_t st) {
+                                   int max_Vp, size_t smem, bool tiled, bool checked, float2* out_one,
+                                   float2* const* d_outs, cudaStream_t st) {
   if (n_entries == 0) return cudaSuccess;
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -815,13 +823,13 @@ cudaError_t launch_recompose_fused(const ItemDev& one, const ItemDev* items, con
   }
   const long long grid = whole + (tiles - whole) * ysplit;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-#define SCW_FU(B, T, G)                                                                                          \
-  [&]() -> cudaError_t {                                                                                         \
-    cudaError_t e = allow_max_smem(reinterpret_cast<const void*>(recompose_fused_kernel<B, T, G>));              \
-    if (e != cudaSuccess) return e;                                                                              \
-    return launch_pdl(recompose_fused_kernel<B, T, G>, dim3((unsigned)grid), dim3(kYregThreads), smem, st, one,   \
-                      items, d_entries, (int)whole, ysplit, out_one, d_outs);                                    \
-  }()
+  auto run = [&](auto kernel) -> cudaError_t {
+    cudaError_t e = allow_max_smem(reinterpret_cast<const void*>(kernel));
+    if (e != cudaSuccess) return e;
+    return launch_pdl(kernel, dim3((unsigned)grid), dim3(kYregThreads), smem, st, one, items, d_entries, (int)whole, ysplit,
+                      out_one, d_outs);
+  };
+#define SCW_FU(B, T, G) (checked ? run(recompose_fused_kernel<B, T, G, true>) : run(recompose_fused_kernel<B, T, G, false>))
 #define SCW_FG(B, T) (ngm == 2 ? SCW_FU(B, T, 2) : ngm == 3 ? SCW_FU(B, T, 3) : SCW_FU(B, T, 6))
   if (items) return tiled ? SCW_FG(true, true) : SCW_FG(true, false);
   return tiled ? SCW_FG(false, true) : SCW_FG(false, false);
