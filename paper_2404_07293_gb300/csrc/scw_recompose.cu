@@ -318,37 +318,37 @@ __device__ __forceinline__ bool y_field_base(const ItemDev& it, int f, int c, in
 }
 
 // One warp's share of a (64-column block, item-plane, component) tile of the y-pass: the residues
-// sub, sub + rs, ... of its columns.
+// sub, sub + rs, ... of its column pairs.
 template <int NG, bool TILED>
 __device__ __forceinline__ void ypass_reg_tile(const ItemDev& it, const float4* tw, int f, int c, int xb, int sub,
                                                int rs, float2* out) {
-  constexpr int COLS = y_cols<NG>();
-  typedef typename ColVec<COLS>::T VecT;
-#pragma unroll 1
-  for (int h = 0; h < 2 / COLS; ++h) {  // COLS 1: the two 32-column halves in turn
-    const int x = xb + 32 * h + COLS * (threadIdx.x & 31);
-    if (x >= it.Fx) return;  // Fx is a multiple of 8: a column pair is in or out as a whole
-    int V = it.V, Fx = it.Fx;
-    // opaque to the compiler: the 8 NG row offsets below are invariant over the tiles, and keeping them
-    // across the loop spills the registers the columns need
-    asm volatile("" : "+r"(V), "+r"(Fx));
-    const size_t tbase = ((size_t)f * 3 + c) * V * Fx + x;
-    VecT d[8 * NG];
+  static_assert(y_cols<NG>() == 2, "a column pair per thread");
+  const int x = xb + 2 * (threadIdx.x & 31);
+  if (x >= it.Fx) return;  // Fx is a multiple of 8: a column pair is in or out as a whole
+  int V = it.V, Fx = it.Fx;
+  // opaque to the compiler: the 8 NG row offsets below are invariant over the tiles, and keeping them
+  // across the loop spills the registers the columns need
+  asm volatile("" : "+r"(V), "+r"(Fx));
+  const size_t tbase = ((size_t)f * 3 + c) * V * Fx + x;
+  float4 d[8 * NG];
 #pragma unroll
-    for (int p = 0; p < 8 * NG; ++p) {
-      const int v = fold_order(p, V, 8 * NG);
-      const size_t i = tbase + (size_t)(max(v, 0) * Fx);  // V Fx <= 96 * 4096
-      d[p] = VecT();
-      if (v >= 0 && in_bounds(it, BND_T, i + COLS - 1)) d[p] = *reinterpret_cast<const VecT*>(it.T + i);
-    }
-    long long obase;
-    if (!y_field_base(it, f, c, x, COLS, obase)) return;
-    y_fold_store<NG, COLS, TILED>(it, d, tw, sub, rs, it.Fy >> 3, out + obase);
+  for (int p = 0; p < 8 * NG; ++p) {
+    const int v = fold_order(p, V, 8 * NG);
+    const size_t i = tbase + (size_t)(max(v, 0) * Fx);  // V Fx <= 24 * 4096
+    d[p] = float4();
+    if (v >= 0 && in_bounds(it, BND_T, i + 1)) d[p] = *reinterpret_cast<const float4*>(it.T + i);
   }
+  long long obase;
+  if (!y_field_base(it, f, c, x, 2, obase)) return;
+  y_fold_store<NG, 2, TILED>(it, d, tw, sub, rs, it.Fy >> 3, out + obase);
 }
 
 constexpr int kYregThreads = 128;
-constexpr int kYregMaxVp = 48;  // longer folds run the shared-memory form (ypass_kernel)
+// Longer folds run the shared-memory form (ypass_kernel): they leave registers for one column per thread, and at
+// 32 to 48 positions the register form is the slower one nearly everywhere (whole step, 9 orders along x, shared ->
+// register, us: 32 positions, 264 x 264 pixels and 16 planes 26.8 -> 30.9, 512 x 128 and 64 planes 51.3 -> 61.6; 48
+// positions 33.0 -> 41.4, 79.7 -> 96.3; it wins at 512 x 512 and 16 planes, 48.0 -> 41.4 and 67.8 -> 65.7).
+constexpr int kYregMaxVp = 24;
 
 // y-pass with the columns in registers. The shared-memory form reads each of the fold's Vp values once
 // per residue (Fy / 8 times): 144 shared-memory wavefronts per 64 columns and residue at Vp = 24, as
@@ -389,9 +389,6 @@ __global__ void __launch_bounds__(kYregThreads, NGM <= 2 ? 4 : 3)
       case 1: ypass_reg_tile<1, TILED>(it, tw, e.y, c, xb, sub, rs, out); break;
       case 2: ypass_reg_tile<2, TILED>(it, tw, e.y, c, xb, sub, rs, out); break;
       case 3: if constexpr (NGM >= 3) ypass_reg_tile<3, TILED>(it, tw, e.y, c, xb, sub, rs, out); break;
-      case 4: if constexpr (NGM >= 6) ypass_reg_tile<4, TILED>(it, tw, e.y, c, xb, sub, rs, out); break;
-      case 5: if constexpr (NGM >= 6) ypass_reg_tile<5, TILED>(it, tw, e.y, c, xb, sub, rs, out); break;
-      case 6: if constexpr (NGM >= 6) ypass_reg_tile<6, TILED>(it, tw, e.y, c, xb, sub, rs, out); break;
     }
   }
   if (one.trace) {
@@ -409,6 +406,7 @@ __global__ void __launch_bounds__(kYregThreads, NGM <= 2 ? 4 : 3)
 // 4096 slots of 128 x 128 680 -> 685 -> 560; a sweep of 32 items 1180 -> 1200 -> 1105. At 256^3 it takes 72 us,
 // 5.6 TB/s of field; packed FP32x2 arithmetic in the y-direction did not change that.
 constexpr int kFusedMaxFx = 256;
+constexpr int kFusedMaxVp = 48;  // orders along y that a thread's column holds in registers
 
 static size_t fused_smem_bytes(int U, int V, int Fx, int Fy) {
   const int Up = fold_np(U), Vp = fold_np(V);
@@ -738,7 +736,8 @@ static cudaError_t launch_ypass_long(const ItemDev& one, const ItemDev* items, c
 
 template <bool BATCH, bool TILED, bool STW, int NGM>
 static cudaError_t launch_ypass_reg(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
-                                    int max_Qx, int tw_f4, float2* out_one, float2* const* d_outs, cudaStream_t st) {
+                                    int max_Qx, int max_Qy, int tw_f4, float2* out_one, float2* const* d_outs,
+                                    cudaStream_t st) {
   const int nxb = (max_Qx * 8 + 63) / 64;
   const long long tiles = (long long)nxb * n_entries * 3;
   const size_t smem = STW ? (size_t)tw_f4 * sizeof(float4) : 0;
@@ -752,6 +751,10 @@ static cudaError_t launch_ypass_reg(const ItemDev& one, const ItemDev* items, co
   // warps per tile: fewer read each x-pass row fewer times, more even out the last round
   int rs = 4;
   while (rs > 1 && tiles * (rs / 2) >= 8 * warps) rs /= 2;
+  // a share of 24 orders reads as much as four output rows of a residue each: short columns take fewer shares as
+  // soon as every warp has one (24 positions, batches of eight items, 4 warps per tile -> this, the shared-memory
+  // form in brackets: 264 x 64 41.2 -> 39.3 us [39.1], 512 x 128 59.8 -> 56.0 [57.6], 1024 x 64 76.4 -> 65.9 [71.8])
+  while (NGM > 2 && rs > 1 && max_Qy < 8 * rs && tiles * (rs / 2) >= warps) rs /= 2;
   const long long shares = tiles * rs;
   if (shares > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = (int)std::min<long long>((shares + kYregThreads / 32 - 1) / (kYregThreads / 32),
@@ -776,10 +779,11 @@ cudaError_t launch_ypass(const ItemDev& one, const ItemDev* items, const int2* d
     ++n;
   }
   if (e == cudaSuccess && n_entries > n_long) {
-    const int ngm = max_Vp <= 16 ? 2 : (max_Vp <= 24 ? 3 : 6);
-#define SCW_YR(B, T, S, G) \
-  launch_ypass_reg<B, T, S, G>(one, items, d_entries + n_long, n_entries - n_long, max_Qx, tw_f4, out_one, d_outs, st)
-#define SCW_YS(B, T, S) (ngm == 2 ? SCW_YR(B, T, S, 2) : ngm == 3 ? SCW_YR(B, T, S, 3) : SCW_YR(B, T, S, 6))
+    const int max_Qy = max_twy / max_Vp;  // of a single plan; of a batch about the largest
+#define SCW_YR(B, T, S, G)                                                                                       \
+  launch_ypass_reg<B, T, S, G>(one, items, d_entries + n_long, n_entries - n_long, max_Qx, max_Qy, tw_f4, out_one, \
+                               d_outs, st)
+#define SCW_YS(B, T, S) (max_Vp <= 16 ? SCW_YR(B, T, S, 2) : SCW_YR(B, T, S, 3))
     if (items)
       e = tiled ? SCW_YS(true, true, false) : SCW_YS(true, false, false);
     else if (stw)
@@ -796,7 +800,7 @@ cudaError_t launch_ypass(const ItemDev& one, const ItemDev* items, const int2* d
 
 size_t fused_recompose_smem(int U, int V, int Fx, int Fy) {
   const size_t b = fused_smem_bytes(U, V, Fx, Fy);
-  return (Fx > kFusedMaxFx || fold_np(V) > kYregMaxVp || b > 72 * 1024) ? 0 : b;  // three CTAs per SM
+  return (Fx > kFusedMaxFx || fold_np(V) > kFusedMaxVp || b > 72 * 1024) ? 0 : b;  // three CTAs per SM
 }
 
 cudaError_t launch_recompose_fused(const ItemDev& one, const ItemDev* items, const int2* d_entries, int n_entries,
