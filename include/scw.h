@@ -181,7 +181,7 @@ scw_status scw_plan_set_layers(scw_plan_t plan, const void* W, const void* gamma
  *   out  DEVICE complex64 [3][Fz][Fy][Fx], x fastest (component-major).
  * The first call for a given `out` launches the kernels; the second one in a row
  * captures them into a CUDA graph, which it and the later calls with the same `out`
- * replay (one launch).
+ * replay (one launch), until another `out` is captured.
  * scw_plan_set_layers and scw_plan_set_timeout_ns drop the graph. */
 scw_status scw_synthesize(scw_plan_t plan, void* out, void* stream);
 

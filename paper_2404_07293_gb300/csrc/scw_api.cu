@@ -14,6 +14,7 @@
 
 #include "scw_internal.cuh"
 #include "scw_points.cuh"
+#include "scw_replay.h"
 
 namespace scw {
 
@@ -590,8 +591,7 @@ struct scw_plan_s {
   // graph replay
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t gexec = nullptr;
-  const void* graph_key = nullptr;
-  const void* seen_key = nullptr;  // output of the last directly launched call (run_synthesis)
+  ReplayRule replay;
   // timing
   bool timing = false;
   std::vector<cudaEvent_t> tev;
@@ -652,8 +652,7 @@ static void free_plan(scw_plan_t P) {
 static void invalidate_graph(scw_plan_t P) {
   if (P->gexec) cudaGraphExecDestroy(P->gexec);
   P->gexec = nullptr;
-  P->graph_key = nullptr;
-  P->seen_key = nullptr;
+  P->replay.drop();
 }
 
 static scw_status upload_items(scw_plan_t P, cudaStream_t st) {
@@ -815,11 +814,8 @@ static scw_status enqueue_synthesis(scw_plan_t P, float2* out_one, cudaStream_t 
   return SCW_OK;
 }
 
-// Timed launches go out directly (with events between kernels). Otherwise the first call for a given
-// output launches directly, the second one captures the same sequence into a CUDA graph, and it and the
-// later calls replay the graph. Capturing and instantiating takes about 50 us of host time, longer than the
-// kernels of a mid-sized field: a program that brings a new solution (which drops the graph) or a new output
-// with every call never pays it.
+// Timed launches go out directly (with events between kernels); otherwise ReplayRule decides between the
+// launches, the capture of the same sequence into a graph and its replay.
 static scw_status run_synthesis(scw_plan_t P, float2* out_one, cudaStream_t st) {
   int n = 0;
   if (P->timing) {
@@ -828,15 +824,16 @@ static scw_status run_synthesis(scw_plan_t P, float2* out_one, cudaStream_t st) 
     return s;
   }
   const void* key = P->batched ? static_cast<const void*>(P->d_outs) : static_cast<const void*>(out_one);
+  const ReplayRule::Step step = P->replay.next(key);
+  if (step == ReplayRule::LAUNCH) {
+    scw_status s = enqueue_synthesis(P, out_one, st, false, n);
+    if (s != SCW_OK) return s;
+    P->kernels_per_synthesis = n;
+    P->replay.done(step, key);
+    return SCW_OK;
+  }
   cudaError_t e;
-  if (!(P->gexec && P->graph_key == key)) {
-    if (P->seen_key != key) {
-      scw_status s = enqueue_synthesis(P, out_one, st, false, n);
-      if (s != SCW_OK) return s;
-      P->kernels_per_synthesis = n;
-      P->seen_key = key;
-      return SCW_OK;
-    }
+  if (step == ReplayRule::CAPTURE) {
     invalidate_graph(P);
     cudaGraph_t g = nullptr;
     e = cudaStreamBeginCapture(P->cap_stream, cudaStreamCaptureModeThreadLocal);
@@ -854,8 +851,8 @@ static scw_status run_synthesis(scw_plan_t P, float2* out_one, cudaStream_t st) 
       P->gexec = nullptr;
       return cuda_error(e, "cudaGraphInstantiate");
     }
-    P->graph_key = key;
   }
+  P->replay.done(step, key);
   e = cudaGraphLaunch(P->gexec, st);
   if (e != cudaSuccess) return cuda_error(e, "cudaGraphLaunch");
   return SCW_OK;
