@@ -814,6 +814,15 @@ static scw_status enqueue_synthesis(scw_plan_t P, float2* out_one, cudaStream_t 
   return SCW_OK;
 }
 
+// While it lives, this thread's calls are allowed although another thread records a graph in the global mode:
+// instantiating one is refused then, and ends the other thread's capture. A plan's own capture uses its own stream
+// only, so neither disturbs the other.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Timed launches go out directly (with events between kernels); otherwise ReplayRule decides between the
 // launches, the capture of the same sequence into a graph and its replay.
 static scw_status run_synthesis(scw_plan_t P, float2* out_one, cudaStream_t st) {
@@ -834,6 +843,7 @@ static scw_status run_synthesis(scw_plan_t P, float2* out_one, cudaStream_t st) 
   }
   cudaError_t e;
   if (step == ReplayRule::CAPTURE) {
+    RelaxedCapture relaxed;
     invalidate_graph(P);
     cudaGraph_t g = nullptr;
     e = cudaStreamBeginCapture(P->cap_stream, cudaStreamCaptureModeThreadLocal);

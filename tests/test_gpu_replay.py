@@ -38,3 +38,44 @@ def test_two_outputs_in_any_order(precision, cuda_device):
     plan.check()
     plan.close()
     other[0].close()
+
+
+@pytest.mark.parametrize("calls_before", [0, 1, 2])
+def test_another_thread_may_be_capturing(calls_before, cuda_device):
+    """The call that captures (the second in a row) works while another thread records a graph, and leaves it whole."""
+    import threading
+
+    import torch
+    plan, layers = _plan(cuda_device)
+    ref = plan.synthesize().clone()
+    out = torch.zeros_like(ref)
+    theirs, ours = torch.cuda.Stream(), torch.cuda.Stream()
+    ours.wait_stream(torch.cuda.current_stream())
+    for _ in range(calls_before):
+        plan.synthesize(out, stream=ours)
+    x = torch.zeros(16, device=cuda_device)
+    torch.cuda.synchronize()
+    errors = []
+
+    def call():
+        try:
+            plan.synthesize(out, stream=ours)
+        except Exception as e:  # noqa: BLE001 - reported below, after the capture has ended
+            errors.append(e)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(theirs):
+        graph.capture_begin(capture_error_mode="global")
+        x += 1
+        t = threading.Thread(target=call)
+        t.start()
+        t.join()
+        graph.capture_end()
+    assert not errors, errors
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(x, torch.ones_like(x))
+    plan.check()
+    plan.close()
