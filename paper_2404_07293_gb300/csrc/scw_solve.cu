@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "../../include/scw_solve.h"
+#include "scw_first_use.h"
 #include "scw_internal.cuh"
 
 namespace scw {
@@ -681,6 +682,31 @@ scw_status scw_solve(scw_solver_t s, const void* n_vol, const void* p_inc_v, voi
     SCW_CU(cudaGetDevice(&dev));
     const int nw = (int)s->eig.size();
     std::vector<std::string> errs(nw);
+    auto decompose = [&](int w, int l) {
+      auto& k = s->eig[w];
+      const cusolverStatus_t r = cusolverDnXgeev(
+          k.h, k.params, CUSOLVER_EIG_MODE_NOVECTOR, CUSOLVER_EIG_MODE_VECTOR, (int64_t)n, CUDA_C_64F,
+          s->C + (size_t)l * nn, (int64_t)n, CUDA_C_64F, s->lam + (size_t)l * n, CUDA_C_64F, nullptr, 1,
+          CUDA_C_64F, s->P + (size_t)l * nn, (int64_t)n, CUDA_C_64F, k.dwork, s->geev_dbytes, k.hwork.data(),
+          k.hwork.size(), s->info + l);
+      if (r != CUSOLVER_STATUS_SUCCESS)
+        errs[w] = "cusolverDnXgeev failed (cuSOLVER status " + std::to_string((int)r) + ")";
+      return r == CUSOLVER_STATUS_SUCCESS;
+    };
+    // A process's first decomposition on a device runs alone: the library loads its kernels in it, and twice a
+    // process whose workers all made that first call at once did not return from here (cause unknown).
+    static FirstUse first;
+    bool ran = false;
+    const bool first_ok = first.alone(dev, ran, [&] {
+      if (cudaStreamWaitEvent(s->eig[0].st, s->ev_ready, 0) != cudaSuccess) {
+        errs[0] = "worker stream setup";
+        return false;
+      }
+      if (!decompose(0, 0)) return false;
+      if (cudaStreamSynchronize(s->eig[0].st) != cudaSuccess) errs[0] = "first eigendecomposition";
+      return errs[0].empty();
+    });
+    if (!first_ok) return set_error(SCW_ERR_CUDA, errs[0]);
     std::vector<std::thread> th;
     for (int w = 0; w < nw; ++w)
       th.emplace_back([&, w] {
@@ -689,17 +715,8 @@ scw_status scw_solve(scw_solver_t s, const void* n_vol, const void* p_inc_v, voi
           errs[w] = "worker stream setup";
           return;
         }
-        for (int l = w; l < L; l += nw) {
-          const cusolverStatus_t r = cusolverDnXgeev(
-              k.h, k.params, CUSOLVER_EIG_MODE_NOVECTOR, CUSOLVER_EIG_MODE_VECTOR, (int64_t)n, CUDA_C_64F,
-              s->C + (size_t)l * nn, (int64_t)n, CUDA_C_64F, s->lam + (size_t)l * n, CUDA_C_64F, nullptr, 1,
-              CUDA_C_64F, s->P + (size_t)l * nn, (int64_t)n, CUDA_C_64F, k.dwork, s->geev_dbytes, k.hwork.data(),
-              k.hwork.size(), s->info + l);
-          if (r != CUSOLVER_STATUS_SUCCESS) {
-            errs[w] = "cusolverDnXgeev failed (cuSOLVER status " + std::to_string((int)r) + ")";
-            return;
-          }
-        }
+        for (int l = w == 0 && ran ? nw : w; l < L; l += nw)
+          if (!decompose(w, l)) return;
         if (cudaEventRecord(k.done, k.st) != cudaSuccess) errs[w] = "worker event";
       });
     for (auto& t : th) t.join();
