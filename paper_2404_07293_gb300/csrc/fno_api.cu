@@ -50,9 +50,12 @@ struct scw_fno_s {
   float* part_mix[8] = {};  // per layer: the gradient partials are reduced together after the backward pass
   float* part_dw[8] = {};
   size_t scratch_floats = 0;
-  // the backward pass's partial-sum reductions, all run by two launches at its end (per batch size)
-  RedSeg* d_segs = nullptr;
-  int segs_B = -1, segs_lift = 0, nseg = 0, seg_items1 = 0, seg_items2 = 0;
+  // the backward pass's partial-sum reductions, all run by two launches at its end: a table for each form of
+  // the lift backward (the input's address chooses it), made anew when the batch size changes
+  struct RedTable {
+    RedSeg* d_segs = nullptr;
+    int B = -1, nseg = 0, items1 = 0, items2 = 0;
+  } red[2];
   float* loss_d = nullptr, *h_d = nullptr, *rel2_d = nullptr;
   int* d_err = nullptr;
   uint64_t timeout_ns = 2000000000ull;
@@ -94,9 +97,10 @@ static cudaError_t falloc(scw_fno_s* f, void** p, size_t bytes) {
 static void free_all(scw_fno_s* f) {
   for (void* p : f->allocs) cudaFree(p);
   f->allocs.clear();
-  if (f->d_segs) cudaFree(f->d_segs);
-  f->d_segs = nullptr;
-  f->segs_B = -1;
+  for (auto& t : f->red) {
+    if (t.d_segs) cudaFree(t.d_segs);
+    t = {};
+  }
   for (cudaEvent_t ev : f->events) cudaEventDestroy(ev);
   f->events.clear();
 }
@@ -269,25 +273,25 @@ static void reduce_into(std::vector<RedSeg>& segs, const float* part, int rows, 
   segs.push_back(sg);
 }
 
-// Every queued reduction in two launches; the table is uploaded when the batch size or the lift
-// backward's form changes.
-static scw_status reduce_all(scw_fno_s* f, std::vector<RedSeg>& segs, int B, int lift_rows, cudaStream_t st) {
-  if (f->segs_B != B || f->segs_lift != lift_rows) {
-    if (!plan_reduce_segments(segs, f->scratch, f->scratch_floats, f->seg_items1, f->seg_items2))
+// Every queued reduction in two launches; the form's table is uploaded when the batch size changes.
+static scw_status reduce_all(scw_fno_s* f, std::vector<RedSeg>& segs, int B, bool lift_cf, cudaStream_t st) {
+  auto& t = f->red[lift_cf];
+  if (t.B != B) {
+    if (!plan_reduce_segments(segs, f->scratch, f->scratch_floats, t.items1, t.items2))
       return set_error(SCW_ERR_UNSUPPORTED, "reduction scratch too small");
-    if (f->d_segs) cudaFree(f->d_segs);
-    f->d_segs = nullptr;
-    cudaError_t e = cudaMalloc(&f->d_segs, segs.size() * sizeof(RedSeg));
+    if (t.d_segs) cudaFree(t.d_segs);
+    t.d_segs = nullptr;
+    t.B = -1;
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&t.d_segs), segs.size() * sizeof(RedSeg));
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(f->d_segs, segs.data(), segs.size() * sizeof(RedSeg), cudaMemcpyHostToDevice, st);
+      e = cudaMemcpyAsync(t.d_segs, segs.data(), segs.size() * sizeof(RedSeg), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // segs is a local table
     if (e != cudaSuccess) return cuda_error(e, "reduction table");
-    f->nseg = (int)segs.size();
-    f->segs_B = B;
-    f->segs_lift = lift_rows;
+    t.nseg = (int)segs.size();
+    t.B = B;
   }
-  cudaError_t e = launch_reduce_segments(f->d_segs, f->nseg, f->seg_items1, f->seg_items2, st);
-  if (f->seg_items2) ++f->counter;
+  cudaError_t e = launch_reduce_segments(t.d_segs, t.nseg, t.items1, t.items2, st);
+  if (t.items2) ++f->counter;
   return launch_ok(f, e, "partial-sum reductions");
 }
 
@@ -395,9 +399,8 @@ static scw_status forward_backward(scw_fno_s* f, const float2* n, const float2* 
   FNO_TRY(launch_ok(f, launch_lift_bwd<T>(static_cast<const T*>(lift_cf ? f->dZcf[cur] : f->dZcl[cur]), lift_cf, n,
                                           f->part_lift, B, f->S, f->in_grid, f->N, st),
                     "lift backward"));
-  const int lift_rows = lift_bwd_rows(lift_cf, B, f->in_grid);
-  reduce_into(segs, f->part_lift, lift_rows, C * 2 * f->S + C, C * 2 * f->S + C, f->grad + f->off_P);
-  return reduce_all(f, segs, B, lift_rows, st);
+  reduce_into(segs, f->part_lift, lift_bwd_rows(lift_cf, B, f->in_grid), C * 2 * f->S + C, C * 2 * f->S + C, f->grad + f->off_P);
+  return reduce_all(f, segs, B, lift_cf, st);
 }
 
 template <typename T>
