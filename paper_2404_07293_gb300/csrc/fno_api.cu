@@ -38,7 +38,7 @@ struct scw_fno_s {
   void* Vcf[9] = {};        // [Bmax][C][P]
   void* Vcl[9] = {};        // [Bmax][P][C]
   void* Gcl[8] = {};        // GELU'(Z_l) [Bmax][P][C], stored by the training forward
-  float* Vh[8] = {};        // complex [kMaxSplit][Kc/2][Bmax C] (mode-major)
+  float* Vh[8] = {};        // complex [splits][Kc/2][Bmax C] (mode-major); kMaxSplit splits in FP32 mode, one in BF16
   float* GWh = nullptr;     // same shape as one Vh
   void* WT = nullptr;       // [L][C][C]: W_l transposed (tensor-core operand of the backward 1x1)
   void* Wh = nullptr;       // [Bmax C][Kp]
@@ -231,7 +231,7 @@ static scw_status forward(scw_fno_s* f, const float2* n, int B, bool keep_z, cud
     FNO_TRY(launch_ok(f, e, "truncated DFT", CAT_DFT, 2.0 * BC * Kd * f->P));
     // Wh carries the inverse transform's 1/N^2 so that the 1x1 convolution can share its accumulator
     if constexpr (std::is_same<T, __nv_bfloat16>::value)
-      e = launch_mix_tc(false, reinterpret_cast<const float2*>(f->Vh[l]), ks, vstride, ld, at<T>(f->wcopy, f->off_R[l]),
+      e = launch_mix_tc(false, reinterpret_cast<const float2*>(f->Vh[l]), ld, at<T>(f->wcopy, f->off_R[l]),
                         static_cast<T*>(f->Wh), inv_n2, B, f->m, f->Kp, f->d_err, f->timeout_ns, st);
     else
       e = launch_mix_fwd<T>(reinterpret_cast<const float2*>(f->Vh[l]), ks, vstride, ld, at<T>(f->wcopy, f->off_R[l]),
@@ -359,12 +359,12 @@ static scw_status forward_backward(scw_fno_s* f, const float2* n, const float2* 
     const int sb = tc_mix ? mix_dr_blocks(B) : mix_sample_blocks(B);
     if constexpr (tc_mix) {
       // GVh = R^H G and the per-block dR, dc partials on the tensor cores
-      FNO_TRY(launch_ok(f, launch_mix_tc(true, reinterpret_cast<const float2*>(f->GWh), ks, vstride, ld,
+      FNO_TRY(launch_ok(f, launch_mix_tc(true, reinterpret_cast<const float2*>(f->GWh), ld,
                                          at<T>(f->wcopy, f->off_R[l]), static_cast<T*>(f->GVh), 1.f, B, f->m,
                                          f->Kp, f->d_err, f->timeout_ns, st),
                         "mode mixing backward (data)", CAT_MIX, 8.0 * f->m * f->m * C * C * B));
       FNO_TRY(launch_ok(f, launch_mix_dr_tc(reinterpret_cast<const float2*>(f->GWh),
-                                            reinterpret_cast<const float2*>(f->Vh[l]), ks, vstride, ld,
+                                            reinterpret_cast<const float2*>(f->Vh[l]), ld,
                                             f->part_mix[l], B, f->m, f->N, f->d_err, f->timeout_ns, st),
                         "mode mixing backward (weights)", CAT_MIX, 8.0 * f->m * f->m * C * C * B));
     } else {
@@ -510,8 +510,10 @@ scw_status scw_surrogate_create(const scw_fno_desc* d, scw_fno_t* out) {
     A(&f->Vcl[l], act);
   }
   for (int l = 0; l + 1 < f->L; ++l) A(&f->Gcl[l], act);
-  for (int l = 0; l < f->L; ++l) A((void**)&f->Vh[l], (size_t)kMaxSplit * Bm * C * f->Kc * 4);
-  A((void**)&f->GWh, (size_t)kMaxSplit * Bm * C * f->Kc * 4);
+  // partial sums: the SIMT products of FP32 mode split K, the tensor-core DFT does not and leaves two dW partials
+  const size_t dft_parts = f->bf16 ? 1 : kMaxSplit, dw_parts = f->bf16 ? 2 : kMaxSplit;
+  for (int l = 0; l < f->L; ++l) A((void**)&f->Vh[l], dft_parts * Bm * C * f->Kc * 4);
+  A((void**)&f->GWh, dft_parts * Bm * C * f->Kc * 4);
   A(&f->Wh, Bm * C * f->Kp * esz);
   A(&f->GVh, Bm * C * f->Kp * esz);
   for (int i = 0; i < 2; ++i) {
@@ -526,7 +528,7 @@ scw_status scw_surrogate_create(const scw_fno_desc* d, scw_fno_t* out) {
   for (int l = 0; l < f->L; ++l)
     A((void**)&f->part_mix[l], (size_t)mix_sample_blocks(f->Bmax) * ((size_t)f->m * f->m * C * C * 2 + C) * 4);
   A(&f->WT, (size_t)f->L * C * C * esz);
-  for (int l = 0; l < f->L; ++l) A((void**)&f->part_dw[l], ((Bm + 3) / 4) * kMaxSplit * 4 * C * C * 4);
+  for (int l = 0; l < f->L; ++l) A((void**)&f->part_dw[l], ((Bm + 3) / 4) * dw_parts * 4 * C * C * 4);
   A((void**)&f->part_lift, ((Bm * f->in_grid * f->in_grid + 127) / 128) * (C * 2 * f->S + C) * 4);
   // reduction chunks: at most 64 rows of every reduced width, for the projection, the weight
   // gradients of every layer and the lift

@@ -11,7 +11,7 @@
 // (r = 0) or imaginary (r = 1) part:
 //   forward   (Re R, -Im R) for r = 0,   (Im R, Re R) for r = 1,  at (2i, 2i + 1)
 //   backward  (Re R,  Im R) for r = 0,   (-Im R, Re R) for r = 1  (R[k][o][i], o as K)
-// The spectra arrive in FP32 (sum of the DFT's K-split partials) and are split
+// The spectra arrive in FP32 and are split
 // into X = X_hi + X_lo (BF16 each), so each mode takes two MMAs into one FP32
 // accumulator: the products keep the weights' BF16 and nearly FP32 spectra.
 //
@@ -33,7 +33,6 @@ namespace scw {
 namespace fno {
 
 constexpr int kMixRows = 128;
-constexpr int kMaxSplitsUnrolled = 2;  // K-split partials of the spectra loaded in one batch
 constexpr uint32_t kMixABytes = kMixRows * 128u;   // one mode's A (hi or lo): 128 rows x 64 BF16
 constexpr uint32_t kMixBBytes = 64u * 128u;        // one mode's B: 64 rows x 64 BF16
 template <int MODES>
@@ -51,8 +50,7 @@ template <> struct ModeWords<2> { typedef uint2 T; };
 template <> struct ModeWords<4> { typedef uint4 T; };
 
 template <bool CONJ, int MODES>
-__global__ void __launch_bounds__(128 * MODES, 4 / MODES) mix_tc_kernel(const float2* __restrict__ X, int splits,
-                                                        long long split_stride, long long ld,
+__global__ void __launch_bounds__(128 * MODES, 4 / MODES) mix_tc_kernel(const float2* __restrict__ X, long long ld,
                                                         const __nv_bfloat16* __restrict__ R,
                                                         __nv_bfloat16* __restrict__ out, float scale, int B, int Kp,
                                                         int* err, uint64_t timeout_ns) {
@@ -78,7 +76,7 @@ __global__ void __launch_bounds__(128 * MODES, 4 / MODES) mix_tc_kernel(const fl
   pdl_sync();  // the spectra come from the preceding kernels
 
   // Operand loads: a thread stages 8 chunks of A (4 complex values each, one 16-byte chunk of BF16)
-  // and 4 chunks of B. Every load it needs (R's words, then the first K-split partial of its A
+  // and 4 chunks of B. Every load it needs (R's words, then its A
   // chunks) is issued before any value is used: with so little work per CTA the staging is bound
   // by memory round trips.
   constexpr int kThreads = 128 * MODES;
@@ -99,45 +97,18 @@ __global__ void __launch_bounds__(128 * MODES, 4 / MODES) mix_tc_kernel(const fl
       rv[jj][e] = CONJ ? R32[((size_t)(k0 + mm) * C + j) * C + p] : R32[((size_t)(k0 + mm) * C + p) * C + j];
     }
   }
-  // A: the spectra of 128 samples (K-split partials summed)
+  // A: the spectra of 128 samples
   float4 va[kChunks], vb[kChunks];
 #pragma unroll
-  for (int z = 0; z < kMaxSplitsUnrolled; ++z) {
-    if (z >= splits) break;  // uniform
-#pragma unroll
-    for (int j = 0; j < kChunks; ++j) {
-      const int q = threadIdx.x + kThreads * j;
-      const int mm = q >> 10, r = (q >> 3) & (kMixRows - 1), g = q & 7;
-      const int b = b0 + r;
-      float4 pa = make_float4(0.f, 0.f, 0.f, 0.f), pb = pa;
-      if (b < B) {
-        const float4* src = reinterpret_cast<const float4*>(X + (size_t)(k0 + mm) * ld + (size_t)b * C + 4 * g +
-                                                            (size_t)z * split_stride);
-        pa = src[0];
-        pb = src[1];
-      }
-      if (z == 0) {
-        va[j] = pa;
-        vb[j] = pb;
-      } else {
-        va[j].x += pa.x; va[j].y += pa.y; va[j].z += pa.z; va[j].w += pa.w;
-        vb[j].x += pb.x; vb[j].y += pb.y; vb[j].z += pb.z; vb[j].w += pb.w;
-      }
-    }
-  }
-  for (int z = kMaxSplitsUnrolled; z < splits; ++z) {  // more K-split partials than the unrolled ones (rare)
-#pragma unroll
-    for (int j = 0; j < kChunks; ++j) {
-      const int q = threadIdx.x + kThreads * j;
-      const int mm = q >> 10, r = (q >> 3) & (kMixRows - 1), g = q & 7;
-      const int b = b0 + r;
-      if (b < B) {
-        const float4* src = reinterpret_cast<const float4*>(X + (size_t)(k0 + mm) * ld + (size_t)b * C + 4 * g +
-                                                            (size_t)z * split_stride);
-        const float4 pa = src[0], pb = src[1];
-        va[j].x += pa.x; va[j].y += pa.y; va[j].z += pa.z; va[j].w += pa.w;
-        vb[j].x += pb.x; vb[j].y += pb.y; vb[j].z += pb.z; vb[j].w += pb.w;
-      }
+  for (int j = 0; j < kChunks; ++j) {
+    const int q = threadIdx.x + kThreads * j;
+    const int mm = q >> 10, r = (q >> 3) & (kMixRows - 1), g = q & 7;
+    const int b = b0 + r;
+    va[j] = vb[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (b < B) {
+      const float4* src = reinterpret_cast<const float4*>(X + (size_t)(k0 + mm) * ld + (size_t)b * C + 4 * g);
+      va[j] = src[0];
+      vb[j] = src[1];
     }
   }
 #pragma unroll
@@ -260,8 +231,7 @@ constexpr uint32_t kDrBBytes = 64u * 128u * kDrKAtoms;           // [4 atoms][64
 constexpr uint32_t kDrSmem = kDrABytes + kDrBBytes + 1024u;
 
 __global__ void __launch_bounds__(256, 2) mix_dr_tc_kernel(const float2* __restrict__ G, const float2* __restrict__ V,
-                                                           int splits, long long split_stride, long long ld,
-                                                           float* __restrict__ part, int B, int m, int N, int* err,
+                                                           long long ld, float* __restrict__ part, int B, int m, int N, int* err,
                                                            uint64_t timeout_ns) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t mma_bar;
@@ -290,34 +260,19 @@ __global__ void __launch_bounds__(256, 2) mix_dr_tc_kernel(const float2* __restr
   for (int j0 = 0; j0 < kDrItems; j0 += kDrBatch) {
     float2 v[kDrBatch][4], g[kDrBatch][4];
 #pragma unroll
-    for (int j = 0; j < kDrBatch; ++j)
+    for (int j = 0; j < kDrBatch; ++j) {
+      const int q = threadIdx.x + 256 * (j0 + j);
+      const int c = q & (C - 1), sq = (q >> 5) % (kDrSamples / 4), mm = q / (C * kDrSamples / 4);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) v[j][e] = g[j][e] = make_float2(0.f, 0.f);
-#pragma unroll 1
-    for (int z = 0; z < splits; ++z) {
-      float2 va[kDrBatch][4], ga[kDrBatch][4];
-#pragma unroll
-      for (int j = 0; j < kDrBatch; ++j) {
-        const int q = threadIdx.x + 256 * (j0 + j);
-        const int c = q & (C - 1), sq = (q >> 5) % (kDrSamples / 4), mm = q / (C * kDrSamples / 4);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int b = b0 + 4 * sq + e;
-          va[j][e] = ga[j][e] = make_float2(0.f, 0.f);
-          if (b < B) {
-            const size_t off = (size_t)(k0 + mm) * ld + (size_t)b * C + c + (size_t)z * split_stride;
-            va[j][e] = V[off];
-            ga[j][e] = G[off];
-          }
+      for (int e = 0; e < 4; ++e) {
+        const int b = b0 + 4 * sq + e;
+        v[j][e] = g[j][e] = make_float2(0.f, 0.f);
+        if (b < B) {
+          const size_t off = (size_t)(k0 + mm) * ld + (size_t)b * C + c;
+          v[j][e] = V[off];
+          g[j][e] = G[off];
         }
       }
-#pragma unroll
-      for (int j = 0; j < kDrBatch; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          v[j][e].x += va[j][e].x; v[j][e].y += va[j][e].y;
-          g[j][e].x += ga[j][e].x; g[j][e].y += ga[j][e].y;
-        }
     }
 #pragma unroll
     for (int j = 0; j < kDrBatch; ++j) {
@@ -371,16 +326,14 @@ __global__ void __launch_bounds__(256, 2) mix_dr_tc_kernel(const float2* __restr
   if (has_dc) {
     const int o = threadIdx.x & (C - 1), pt = threadIdx.x >> 5;
     float d = 0.f;
-    for (int z = 0; z < splits; ++z) {
-      float x[16];
+    float x[16];
 #pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        const int b = b0 + 16 * pt + e;
-        x[e] = b < B ? G[(size_t)kdc * ld + (size_t)b * C + o + (size_t)z * split_stride].x : 0.f;
-      }
-#pragma unroll
-      for (int e = 0; e < 16; ++e) d += x[e];
+    for (int e = 0; e < 16; ++e) {
+      const int b = b0 + 16 * pt + e;
+      x[e] = b < B ? G[(size_t)kdc * ld + (size_t)b * C + o].x : 0.f;
     }
+#pragma unroll
+    for (int e = 0; e < 16; ++e) d += x[e];
     dc_part[pt][o] = d;
   }
   __syncthreads();
@@ -421,26 +374,25 @@ __global__ void __launch_bounds__(256, 2) mix_dr_tc_kernel(const float2* __restr
 
 int mix_dr_blocks(int B) { return (B + kDrSamples - 1) / kDrSamples; }
 
-cudaError_t launch_mix_dr_tc(const float2* G, const float2* V, int splits, long long split_stride, long long ld,
-                             float* part, int B, int m, int N, int* err, uint64_t timeout_ns, cudaStream_t st) {
+cudaError_t launch_mix_dr_tc(const float2* G, const float2* V, long long ld, float* part, int B, int m, int N, int* err,
+                             uint64_t timeout_ns, cudaStream_t st) {
   if ((m * m) % kDrModes) return cudaErrorInvalidValue;
   const void* fn = reinterpret_cast<const void*>(mix_dr_tc_kernel);
   cudaError_t e = allow_max_smem(fn);
   if (e != cudaSuccess) return e;
   const dim3 grid(m * m / kDrModes, (B + kDrSamples - 1) / kDrSamples);
-  return launch_pdl(mix_dr_tc_kernel, grid, dim3(256), kDrSmem, st, G, V, splits, split_stride, ld, part, B, m, N, err,
+  return launch_pdl(mix_dr_tc_kernel, grid, dim3(256), kDrSmem, st, G, V, ld, part, B, m, N, err,
                     timeout_ns);
 }
 
-cudaError_t launch_mix_tc(bool conj, const float2* X, int splits, long long split_stride, long long ld,
-                          const __nv_bfloat16* R, __nv_bfloat16* out, float scale, int B, int m, int Kp, int* err,
-                          uint64_t timeout_ns, cudaStream_t st) {
-  if ((m * m) % 2 || Kp % 8 || (ld % 2) || (split_stride % 2)) return cudaErrorInvalidValue;
+cudaError_t launch_mix_tc(bool conj, const float2* X, long long ld, const __nv_bfloat16* R, __nv_bfloat16* out,
+                          float scale, int B, int m, int Kp, int* err, uint64_t timeout_ns, cudaStream_t st) {
+  if ((m * m) % 2 || Kp % 8 || (ld % 2)) return cudaErrorInvalidValue;
   const int blocks = (B + kMixRows - 1) / kMixRows;
   auto run = [&](auto kernel, int modes, uint32_t smem) -> cudaError_t {
     cudaError_t e = allow_max_smem(reinterpret_cast<const void*>(kernel));
     if (e != cudaSuccess) return e;
-    return launch_pdl(kernel, dim3(m * m / modes, blocks), dim3(128 * modes), smem, st, X, splits, split_stride, ld, R, out,
+    return launch_pdl(kernel, dim3(m * m / modes, blocks), dim3(128 * modes), smem, st, X, ld, R, out,
                       scale, B, Kp, err, timeout_ns);
   };
   if ((m * m) % 4 == 0 && blocks > 1)
