@@ -399,13 +399,10 @@ int lift_bwd_rows(bool channel_first, int B, int in_grid);
 template <typename T>
 cudaError_t launch_lift_bwd(const T* dV0, bool channel_first, const float2* n, float* part, int B, int S, int in_grid,
                             int N, cudaStream_t st);
-cudaError_t launch_reduce_rows_ex(const float* part, int rows, int width, long long pitch, float scale, float* out,
-                                  float* scratch, cudaStream_t st);
 
 // One deterministic partial-sum reduction out[j] += sum_r part[r pitch + j] of a set, all run by
 // two launches (reduce_segments). Rows above 256 are summed in ry chunks of `chunk` rows into
-// `scratch` ([ry][width]) and the chunks then in a second pass, with the same order of additions
-// as launch_reduce_rows_ex.
+// `scratch` ([ry][width]) and the chunks then in a second pass, so that no thread sums more than about 32.
 struct RedSeg {
   const float* part;
   float* out;

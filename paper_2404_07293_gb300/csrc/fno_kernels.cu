@@ -1090,28 +1090,6 @@ __global__ void __launch_bounds__(256) lift_bwd_mma_kernel(const __nv_bfloat16* 
   }
 }
 
-// ---- deterministic column sums: block (32, 8) per 32 columns and a chunk of rows
-__global__ void __launch_bounds__(256) reduce_rows_kernel(const float* __restrict__ part, int rows, int width,
-                                                          long long pitch, int chunk, float scale,
-                                                          float* __restrict__ out, float* __restrict__ scratch) {
-  __shared__ float red[8][33];
-  const int col = blockIdx.x * 32 + threadIdx.x;
-  const int r0 = blockIdx.y * chunk, r1 = min(rows, r0 + chunk);
-  float s = 0.f;
-  if (col < width)
-    for (int r = r0 + threadIdx.y; r < r1; r += 8) s += part[(size_t)r * pitch + col];
-  red[threadIdx.y][threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.y == 0 && col < width) {
-    float t = 0.f;
-    for (int y = 0; y < 8; ++y) t += red[y][threadIdx.x];
-    if (scratch)
-      scratch[(size_t)blockIdx.y * width + col] = t;
-    else
-      out[col] += scale * t;
-  }
-}
-
 // ---- Adam (bias-corrected), refreshes the kernels' copy of the parameters
 template <typename T>
 __global__ void adam_kernel(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
@@ -1394,7 +1372,8 @@ cudaError_t launch_lift_bwd(const T* dV0, bool channel_first, const float2* n, f
 
 constexpr int kWideCols = 4;  // columns per thread of a segment with few rows (one 16-byte load per row)
 
-// Segmented form of reduce_rows_kernel: block b belongs to the last segment whose first item is <= b
+// ---- deterministic column sums of many segments: block (32, 8) per 32 columns and a chunk of rows (rows above 256
+// go through scratch rows in a second pass). Block b belongs to the last segment whose first item is <= b
 // (every lane of a warp looks at one segment; at most 32 segments).
 __device__ __forceinline__ int find_segment(const RedSeg* segs, int nseg, int b, bool second) {
   const int i = threadIdx.x;  // lane: blocks are (32, 8)
@@ -1492,24 +1471,6 @@ cudaError_t launch_reduce_segments(const RedSeg* d_segs, int nseg, int items1, i
   cudaError_t e = launch_pdl(reduce_segments_kernel, dim3(items1), dim3(32, 8), 0, st, d_segs, nseg, 0);
   if (e != cudaSuccess || items2 == 0) return e;
   return launch_pdl(reduce_segments_kernel, dim3(items2), dim3(32, 8), 0, st, d_segs, nseg, 1);
-}
-
-// out[j] += scale * sum_r part[r pitch + j]; rows above 256 go through `scratch`
-// (64 rows of `width`) in a second pass so that no thread sums more than ~32 rows.
-cudaError_t launch_reduce_rows_ex(const float* part, int rows, int width, long long pitch, float scale, float* out,
-                                  float* scratch, cudaStream_t st) {
-  if (rows <= 0 || width <= 0) return cudaSuccess;
-  const dim3 block(32, 8);
-  const unsigned gx = (unsigned)((width + 31) / 32);
-  if (rows <= 256 || !scratch) {
-    reduce_rows_kernel<<<dim3(gx, 1), block, 0, st>>>(part, rows, width, pitch, rows, scale, out, nullptr);
-    return cudaGetLastError();
-  }
-  const int ry = std::min(64, (rows + 255) / 256);
-  const int chunk = (rows + ry - 1) / ry;
-  reduce_rows_kernel<<<dim3(gx, ry), block, 0, st>>>(part, rows, width, pitch, chunk, scale, out, scratch);
-  reduce_rows_kernel<<<dim3(gx, 1), block, 0, st>>>(scratch, ry, width, width, ry, scale, out, nullptr);
-  return cudaGetLastError();
 }
 
 template <typename T>
