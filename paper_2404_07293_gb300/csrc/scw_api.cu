@@ -219,7 +219,8 @@ static scw_status assign_planes(Plan* p, std::vector<int>& ext, int& max_nf) {
     if (_e != cudaSuccess) return cuda_error(_e, #x); \
   } while (0)
 
-// Tables and every buffer except S_part (whose size depends on the split).
+// Tables and every buffer except S_part (whose size depends on the split) and T (which the one-kernel recomposition
+// does without).
 static scw_status build_item(Plan* p, const std::vector<int>& ext) {
   std::vector<double2> szt(p->M), szb(p->M);
   std::vector<float> pupil(p->M, 1.f);
@@ -263,7 +264,6 @@ static scw_status build_item(Plan* p, const std::vector<int>& ext) {
   if (p->pupil_na > 0) SCW_TRY(upload(&p->d_pupil, pupil, tot));
   SCW_TRY(upload(&p->d_twx, twx, tot));
   SCW_TRY(upload(&p->d_twy, twy, tot));
-  SCW_TRY(dalloc(&p->T, (size_t)p->Fz * 3 * p->V * p->Fx, tot));
   if (n_units > 0) {
     if (p->precision == SCW_PREC_FP32) {
       SCW_TRY(dalloc(&p->Wt, L * 3 * M * 4 * M, tot));
@@ -295,6 +295,13 @@ static scw_status build_item(Plan* p, const std::vector<int>& ext) {
   }
   SCW_TRY(cudaEventCreate(&p->ev0));
   SCW_TRY(cudaEventCreate(&p->ev1));
+  return SCW_OK;
+}
+
+// The x-pass rows.
+static scw_status alloc_rows(Plan* p) {
+  if (!p->T) SCW_TRY(dalloc(&p->T, (size_t)p->Fz * 3 * p->V * p->Fx, p->workspace_bytes));
+  p->item.T = p->T;
   return SCW_OK;
 }
 
@@ -1056,6 +1063,11 @@ static scw_status finish_plan(scw_plan_t P, const std::vector<int>& user_ks, boo
   P->n_long_entries = 0;
   for (const int2& en : pe) P->n_long_entries += ypass_long(P->items[en.x]->item.Vp) ? 1 : 0;
   P->fused_smem = fuse_recompose(P, (int)pe.size());
+  for (auto* p : P->items)
+    if (!P->fused_smem || P->checked || (p->flags & SCW_FLAG_HOST_IO)) {
+      scw_status s = alloc_rows(p);
+      if (s != SCW_OK) return s;
+    }
   P->phase.max_M = P->max_M;
   P->phase.F_pad = P->F_pad;
   P->n_unit_entries = (int)ue.size();
@@ -1743,6 +1755,11 @@ scw_status scw_plan_set_pipeline(scw_plan_t P, int groups) {
   invalidate_graph(P);
   P->groups = groups;
   if (groups == 1) return SCW_OK;
+  scw_status rs = alloc_rows(p);  // the groups run the x-pass and the y-pass
+  if (rs != SCW_OK) {
+    P->groups = 1;
+    return rs;
+  }
   cudaError_t e;
   if (!P->st2) {
     e = cudaStreamCreateWithFlags(&P->st2, cudaStreamNonBlocking);

@@ -75,3 +75,25 @@ def test_checked_batch_runs_every_form(cuda_device):
     assert kernels[1] == kernels[0] + 3  # the x-pass and, for 16 to 32 fold positions, both y-pass kernels
     for a, b in zip(*outs):
         assert torch.equal(a, b)
+
+
+def test_rows_are_allocated_where_a_kernel_writes_them(cuda_device):
+    """The x-pass rows [planes][3][V][Fx] belong to plans that run the x-pass."""
+    shape = (9, 9, 136, 64, 40)
+    rows = 40 * 3 * 9 * 136 * 8
+    plan = _plan(*shape, cuda_device)
+    fused = plan.info()["workspace_bytes"]
+    ref = plan.synthesize()
+    plan.set_pipeline(2)
+    assert plan.info()["workspace_bytes"] == fused + rows
+    out = plan.synthesize()
+    plan.set_pipeline(1)
+    plan.set_pipeline(2)
+    assert plan.info()["workspace_bytes"] == fused + rows
+    plan.check()
+    assert (out == ref).all()
+    plan.close()
+    for extra in (dict(debug_bounds=True), dict(host_io=True)):
+        with_rows = _plan(*shape, cuda_device, **extra)
+        assert with_rows.info()["workspace_bytes"] >= fused + rows
+        with_rows.close()
