@@ -383,15 +383,25 @@ static scw_status finish_item(Plan* p) {
   return SCW_OK;
 }
 
+// Layers and plane slots of a descriptor. I illuminations share every plane: slot f I + i is output plane f of
+// illumination i.
+static void plane_slots(Plan* p, const scw_desc* d) {
+  p->L = d->L;
+  p->I = std::max(1, d->illuminations);
+  p->Fz_out = d->Fz;
+  p->Fz = p->I * d->Fz;
+  p->z_bounds.assign(d->z_bounds, d->z_bounds + d->L + 1);
+  p->z_planes.clear();
+  for (int f = 0; f < d->Fz; ++f)
+    for (int i = 0; i < p->I; ++i) p->z_planes.push_back(d->z_planes[f]);
+}
+
 static scw_status create_item(const scw_desc* d, int force_F_pad, Plan** out) {
   *out = nullptr;
   Plan* p = new (std::nothrow) Plan();
   if (!p) return set_error(SCW_ERR_OUT_OF_MEMORY, "host allocation failed");
-  p->U = d->U; p->V = d->V; p->M = d->U * d->V; p->L = d->L;
-  // I illuminations share every plane: plane slot f I + i is output plane f of illumination i
-  p->I = std::max(1, d->illuminations);
-  p->Fz_out = d->Fz;
-  p->Fx = d->Fx; p->Fy = d->Fy; p->Fz = p->I * d->Fz;
+  p->U = d->U; p->V = d->V; p->M = d->U * d->V;
+  p->Fx = d->Fx; p->Fy = d->Fy;
   p->pupil_na = d->pupil_na;
   p->tiles_x = std::max(1, d->tiles_x);
   p->tiles_y = std::max(1, d->tiles_y);
@@ -400,10 +410,7 @@ static scw_status create_item(const scw_desc* d, int force_F_pad, Plan** out) {
   p->lambda = d->lambda; p->X = d->X; p->Y = d->Y; p->x0 = d->x0; p->y0 = d->y0;
   p->n_top = d->n_top; p->n_bot_re = d->n_bot_re; p->n_bot_im = d->n_bot_im; p->z_inc = d->z_inc;
   p->precision = d->precision; p->flags = d->flags;
-  p->z_bounds.assign(d->z_bounds, d->z_bounds + d->L + 1);
-  p->z_planes.clear();
-  for (int f = 0; f < d->Fz; ++f)
-    for (int i = 0; i < p->I; ++i) p->z_planes.push_back(d->z_planes[f]);
+  plane_slots(p, d);
   std::vector<int> ext;
   int max_nf = 0;
   scw_status s = assign_planes(p, ext, max_nf);
@@ -1352,11 +1359,8 @@ scw_status scw_plan_batched(const scw_desc* descs, int n, void* stream, scw_plan
   int fpad = 8;
   for (int i = 0; i < n; ++i) {
     Plan probe;
-    probe.L = descs[i].L;
-    probe.Fz = descs[i].Fz;
     probe.flags = descs[i].flags | SCW_FLAG_EXTERIOR;
-    probe.z_bounds.assign(descs[i].z_bounds, descs[i].z_bounds + descs[i].L + 1);
-    probe.z_planes.assign(descs[i].z_planes, descs[i].z_planes + descs[i].Fz);
+    plane_slots(&probe, &descs[i]);
     std::vector<int> ext;
     int max_nf = 0;
     assign_planes(&probe, ext, max_nf);
