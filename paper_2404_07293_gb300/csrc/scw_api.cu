@@ -516,8 +516,8 @@ static scw_status check_task_ranges(const Plan* p, const int4& tk) {
   const size_t s_end = ((size_t)tk.w * p->Fz + u.f0 + u.nf - 1) * R + (size_t)p->rows_tile * tk.z + rt;
   std::string why;
   if (rt <= 0 || tk.w >= ks || u.layer < 0 || u.layer >= p->L) why = "its row tile, split or layer";
-  else if (a_end > (size_t)p->L * R * nk * 64) why = "W";
-  else if (b_end > p->units.size() * (size_t)nk * p->NB * 64) why = "the B operand";
+  else if (kcount > 0 && a_end > (size_t)p->L * R * nk * 64) why = "W";  // (an empty split copies nothing and stores zeros)
+  else if (kcount > 0 && b_end > p->units.size() * (size_t)nk * p->NB * 64) why = "the B operand";
   else if (s_end > (size_t)p->k_split * p->Fz * R) why = "the partial spectra";
   if (why.empty()) return SCW_OK;
   return set_error(SCW_ERR_BOUNDS, "contraction task (unit " + std::to_string(tk.y) + ", tile " + std::to_string(tk.z) +

@@ -97,3 +97,22 @@ def test_rows_are_allocated_where_a_kernel_writes_them(cuda_device):
         with_rows = _plan(*shape, cuda_device, **extra)
         assert with_rows.info()["workspace_bytes"] >= fused + rows
         with_rows.close()
+
+
+@pytest.mark.parametrize("precision", ["split_bf16", "fp16"])
+@pytest.mark.parametrize("U,V,planes,k_split", [(23, 24, 16, 0), (5, 5, 16, 3), (9, 9, 24, 8), (4, 4, 30, 16)])
+def test_checked_plan_with_an_empty_split(U, V, planes, k_split, precision, cuda_device):
+    """K splits that leave the last one without a chunk (nk chunks in ceil(nk / k) per split) are no violation."""
+    import torch
+    import paper_2404_07293_gb300 as scw
+    W, g, a, *_ = wl.random_layer_set(U + V, U, V, 2)
+    fields = []
+    for debug in (False, True):
+        plan = scw.Plan(U=U, V=V, L=2, lam=1.0, X=3.1, Y=2.7, z_bounds=np.array([0.0, 0.4, 0.7]), Fx=64, Fy=32,
+                        z_planes=wl.cell_centred_planes(0.0, 0.7, planes), precision=precision, k_split=k_split,
+                        debug_bounds=debug)
+        plan.set_layers(*(torch.from_numpy(np.ascontiguousarray(x)).to(cuda_device) for x in (W, g, a)))
+        fields.append(plan.synthesize())
+        plan.check()
+        plan.close()
+    assert torch.equal(*fields)
