@@ -121,7 +121,9 @@ __global__ void __launch_bounds__(128, FCH == 8 ? 4 : 3)
 // Modes in which W^T is split over CTAs: the split with the shortest schedule, rounds of resident CTAs (four
 // per SM up to 8 planes, three above) of K / ks modes each plus about 24 modes' worth of start and end. At
 // most kMaxChain modes are summed in one FP32 chain: longer ones saved 5 us of 213 at 21 x 21 orders and
-// 32 layers, but raised the field's error against 64 bits from 4.4e-7 to 6.7e-7.
+// 32 layers, but raised the field's error against 64 bits from 4.4e-7 to 6.7e-7. The partial spectra grow with the
+// splits: 64 x 64 orders, 2 layers of 16 planes take 64 (201 MB beside 6.4 GB of W and W^T) where chains of 768 modes
+// took 22; writing and adding them is part of that step's 1046 us (2795 with the chains and without loads in flight).
 constexpr int kMaxChain = 256;
 
 int fp32_split(int n_units, int M, int F_pad, int sms) {

@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(192) contract_tc_kernel(const __grid_constant_
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t_begin = cta_off[blockIdx.x], t_end = cta_off[blockIdx.x + 1];
   const uint64_t deadline = ptx::globaltimer() + timeout_ns;
-  ptx::griddep_launch_dependents();  // the x-pass may be scheduled as CTAs of this grid finish
+  ptx::griddep_launch_dependents();  // the recomposition may be scheduled as CTAs of this grid finish
   trace_begin(one.trace, TRACE_CONTRACT);
 
   if (threadIdx.x == 0) {
@@ -318,9 +318,9 @@ __global__ void __launch_bounds__(192) contract_tc_kernel(const __grid_constant_
 // 0.8. So A and B have rings of their own, and B's is cut into halves of 128 columns, multiplied one after
 // the other (N = 128): four half chunks of B and three chunks of A (from memory) are in flight, and a half is
 // requested again as soon as its own MMAs are done. The same products in the same order. 16 illuminations
-// at 21 x 21 orders, 32 layers of 8 planes: 174 -> 161 us, 91 % of the tensor cores' rate under the power
-// cap. (Two row tiles per task, so that a B chunk is used twice, leave no tensor memory for a second set of
-// accumulators: 191 us.)
+// at 21 x 21 orders, 32 layers of 8 planes: 174 -> 161 us, 1425 TFLOP/s of the three products, 0.84 of the tensor
+// cores' rate under the power cap (0.91 with padded rows and K counted). (Two row tiles per task, so that a B chunk
+// is used twice, leave no tensor memory for a second set of accumulators: 191 us.)
 template <bool SPLIT>
 struct RingCfg {
   static constexpr int NB = 256, HB = 128;
