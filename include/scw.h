@@ -80,7 +80,8 @@ enum {
   SCW_FLAG_AUTOTUNE = 4u, /* time the best contraction schedules on the device at plan
                              creation (otherwise a makespan model picks the split);
                              results are cached per device and problem shape           */
-  SCW_FLAG_DEBUG_BOUNDS = 8u /* index checks: every kernel of the plan compares each global
+  SCW_FLAG_DEBUG_BOUNDS = 8u /* index checks: every kernel of scw_synthesize (not those of
+                             scw_recompose and of the point sets) compares each global
                              index it forms (spectra, x-pass rows, twiddles, B operand,
                              gamma/alpha, the FP32 path's operands, the field) with the
                              extent of its buffer; an index outside is not accessed, the
