@@ -406,10 +406,10 @@ __global__ void __launch_bounds__(kYregThreads, NGM <= 2 ? 4 : 3)
 // shared-memory y-pass -> x-pass and register y-pass -> this kernel: 256^3 192.6 -> 189.5 -> 179.3 us;
 // 4096 slots of 128 x 128 680 -> 685 -> 560; a sweep of 32 items 1180 -> 1200 -> 1105. At 256^3 it takes 72 us,
 // 5.6 TB/s of field; packed FP32x2 arithmetic in the y-direction did not change that.
-// Wider rows (the x-direction's loop takes up to 1024 pixels) gain with short columns and lose with tall ones, where
-// the columns of a plane no longer come out even over the CTA's threads: one kernel against two, us of a whole step,
-// 21 orders, 264 x 64 and 128 planes 35.1 / 45.2, 264 x 512 and 24 planes 39.1 / 35.0; 15 orders, 264 x 512 and 24
-// planes 35.0 / 30.9; 7 orders, 1024 x 512 and 24 planes 77.7 / 63.9. Median of 80 shapes 0.99.
+// Wider rows (the x-direction's loop takes up to 1024 pixels) gain with short columns and lose with tall ones: one
+// kernel against two, us of a whole step, 21 orders, 264 x 64 and 128 planes 35.1 / 45.2, 264 x 512 and 24 planes
+// 39.1 / 35.0; 15 orders, 264 x 512 and 24 planes 35.0 / 30.9; 7 orders, 1024 x 512 and 24 planes 77.7 / 63.9. Over
+// 80 shapes the median is 0.99 of the two kernels' time.
 constexpr int kFusedMaxFx = 256;
 constexpr int kFusedMaxVp = 48;  // orders along y that a thread's column holds in registers
 
